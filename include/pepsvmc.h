@@ -109,12 +109,13 @@ int pepsvmc_get_spins(pepsvmc_ctx* ctx, int8_t* spins);
 int pepsvmc_set_tensors(pepsvmc_ctx* ctx, const double* tensors);
 int pepsvmc_get_tensors(pepsvmc_ctx* ctx, double* tensors);
 
-/* Fused three-line steps (on by default in the BF16 and split-BF16 precisions): the
- * three products of a column step (App. C) run in one tensor-core kernel per chain and
- * bond tile, with the intermediates kept in tensor and shared memory; bonds up to
- * Dc = 32 and D = 8, larger ones use the separate products.  pepsvmc_set_fused(ctx, 0)
- * computes every step as three separate products (same arithmetic type, other
- * rounding order).  Forcing a contraction kernel (pepsvmc_set_contraction_kernel)
+/* Fused column steps (on by default).  In the BF16 and split-BF16 precisions the products
+ * of a column step (App. C) run in one tensor-core kernel per chain and bond tile, with the
+ * intermediates kept in tensor and shared memory, for bonds up to Dc = 32 and D = 8; in FP32
+ * they run in one CUDA-core kernel with the intermediates in shared memory, as far as
+ * those fit.  Larger steps, and TF32, use the separate products.
+ * pepsvmc_set_fused(ctx, 0) computes every step as separate products (same arithmetic type;
+ * tensor-core results in another rounding order, FP32 results with the same bits).  Forcing a contraction kernel (pepsvmc_set_contraction_kernel)
  * also disables the fused steps.  Drops a captured step graph.                  */
 int pepsvmc_set_fused(pepsvmc_ctx* ctx, int32_t on);
 

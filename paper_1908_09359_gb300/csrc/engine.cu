@@ -22,6 +22,7 @@
 
 #include "common.cuh"
 #include "fused.cuh"
+#include "fused_f32.cuh"
 #include "kernels.cuh"
 #include "pepsvmc.h"
 #include "proposal.cuh"
@@ -474,20 +475,22 @@ struct pepsvmc_ctx {
     return fused_on && forced < 0 && (tc_mode() == 2 || tc_mode() == 3) &&
            env3_fused_fits(cT, cB, cT2, cB2, a.Dl, a.Dr, a.Du, a.Dd);
   }
+  bool spans3(const Env3Fused& f) {
+    const long long b1 = f.batch - 1;
+    return span(f.E, b1 * f.bsE + (f.cT - 1) * f.sEa + (f.Dl - 1) * f.sEl + (f.cB - 1) * f.sEb, 4, "fused E") &&
+           span(f.T, b1 * f.bsT + (f.cT - 1) * f.sTa + (f.Du - 1) * f.sTu + (f.cT2 - 1) * f.sTa2, 4, "fused T") &&
+           span(f.A, f.ssA + (f.Dl - 1) * f.sAl + (f.Du - 1) * f.sAu + (f.Dr - 1) * f.sAr + (f.Dd - 1) * f.sAd, 4,
+                "fused A") &&
+           span(f.B, b1 * f.bsB + (f.cB - 1) * f.sBb + (f.Dd - 1) * f.sBd + (f.cB2 - 1) * f.sBb2, 4, "fused B") &&
+           span(f.out, b1 * f.bsO + (f.cT2 - 1) * f.sOa2 + (f.Dr - 1) * f.sOr + (f.cB2 - 1) * f.sOb2, 4, "fused out") &&
+           (!f.sel || span(f.sel, b1 * f.sel_stride, 1, "fused spin selector"));
+  }
   // caller_memory: the operands are the caller's (the C-ABI step), not the context's
   // allocations, so the context's bounds table does not cover them
   cudaError_t fused3(Env3Fused f, int batch = 0, bool caller_memory = false) {
     f.batch = batch > 0 ? batch : C;
     f.wait_cycles = wait_budget;
-    const long long b1 = f.batch - 1;
-    if (!caller_memory && (!span(f.E, b1 * f.bsE + (f.cT - 1) * f.sEa + (f.Dl - 1) * f.sEl + (f.cB - 1) * f.sEb, 4, "fused E") ||
-        !span(f.T, b1 * f.bsT + (f.cT - 1) * f.sTa + (f.Du - 1) * f.sTu + (f.cT2 - 1) * f.sTa2, 4, "fused T") ||
-        !span(f.A, f.ssA + (f.Dl - 1) * f.sAl + (f.Du - 1) * f.sAu + (f.Dr - 1) * f.sAr + (f.Dd - 1) * f.sAd, 4,
-              "fused A") ||
-        !span(f.B, b1 * f.bsB + (f.cB - 1) * f.sBb + (f.Dd - 1) * f.sBd + (f.cB2 - 1) * f.sBb2, 4, "fused B") ||
-        !span(f.out, b1 * f.bsO + (f.cT2 - 1) * f.sOa2 + (f.Dr - 1) * f.sOr + (f.cB2 - 1) * f.sOb2, 4, "fused out") ||
-        (f.sel && !span(f.sel, b1 * f.sel_stride, 1, "fused spin selector"))))
-      return cudaErrorInvalidValue;
+    if (!caller_memory && !spans3(f)) return cudaErrorInvalidValue;
     ++launches;
     const double nb = f.batch;
     const double flops = 2.0 * nb *
@@ -537,23 +540,79 @@ struct pepsvmc_ctx {
     return f;
   }
 
+  // FP32 three-line step in one kernel (intermediates in shared memory): the same sums in the
+  // same order as the separate products (rev: those of the right step).  out1: the result with
+  // the other slot of the site, sharing E . T.
+  bool f32_fused() const { return fused_on && forced < 0 && tc_mode() == 0; }
+  bool f32_ok(const Env3Fused& f) const { return f32_fused() && env3_f32_fits(f); }
+  cudaError_t step3_f32(Env3Fused f, float* out1, bool rev, int batch = 0, bool caller_memory = false) {
+    f.batch = batch > 0 ? batch : C;
+    if (!caller_memory) {
+      Env3Fused g = f;
+      g.out = out1 ? out1 : f.out;
+      if (!spans3(f) || !spans3(g)) return cudaErrorInvalidValue;
+    }
+    ++launches;
+    const double nb = f.batch, nv = out1 ? 2.0 : 1.0;
+    const double flops = 2.0 * nb *
+        ((double)f.Dl * f.cB * f.Du * f.cT2 * f.cT +
+         nv * ((double)f.cB * f.cT2 * f.Dr * f.Dd * f.Dl * f.Du + (double)f.cT2 * f.Dr * f.cB2 * f.cB * f.Dd));
+    if (prof) {
+      prof_acc[0] += 1;
+      prof_acc[1] += flops;
+      prof_acc[5] += 4.0 * ((f.bsE ? nb : 1.0) * f.cT * f.Dl * f.cB + (f.bsT ? nb : 1.0) * f.cT * f.Du * f.cT2 +
+                            (f.bsB ? nb : 1.0) * f.cB * f.Dd * f.cB2 + nv * nb * f.cT2 * f.Dr * f.cB2 +
+                            2.0 * f.Dl * f.Du * f.Dr * f.Dd);
+    }
+    char key[96];
+    snprintf(key, sizeof(key), "step3 f32 %d %d %d %d x %d %d %d %d", f.cT, f.cB, f.cT2, f.cB2, f.Dl, f.Dr, f.Du, f.Dd);
+    return timed(0, [&] { return env3_f32(f, out1, rev, st); }, key, flops);
+  }
+  // FP32 four-line step, one to four flip variants (see Env4Outs) of it in one kernel.
+  cudaError_t step4_f32(Env4Fused f, const Env4Outs& o, bool rev) {
+    f.batch = C;
+    for (float* p : o.p) {
+      f.out = p;
+      if (p && !spans4(f)) return cudaErrorInvalidValue;
+    }
+    ++launches;
+    const double nb = C, s1 = (double)f.D1l * f.D2l * f.cB * f.Du1 * f.cT2 * f.cT,
+                 s2 = (double)f.D2l * f.cB * f.cT2 * f.D1r * f.Dd1 * f.D1l * f.Du1,
+                 s34 = (double)f.cB * f.cT2 * f.D1r * f.D2r * f.Dd2 * f.D2l * f.Dd1 +
+                       (double)f.cT2 * f.D1r * f.D2r * f.cB2 * f.cB * f.Dd2;
+    const int n0 = (o.p[0] != nullptr) + (o.p[1] != nullptr), n1 = (o.p[2] != nullptr) + (o.p[3] != nullptr);
+    const double flops = 2.0 * nb * (s1 + ((n0 > 0) + (n1 > 0)) * s2 + (n0 + n1) * s34);
+    if (prof) {
+      prof_acc[0] += 1;
+      prof_acc[1] += flops;
+      prof_acc[5] += 4.0 * ((f.bsE ? nb : 1.0) * f.cT * f.D1l * f.D2l * f.cB + (f.bsT ? nb : 1.0) * f.cT * f.Du1 * f.cT2 +
+                            (f.bsB ? nb : 1.0) * f.cB * f.Dd2 * f.cB2 + (n0 + n1) * nb * f.cT2 * f.D1r * f.D2r * f.cB2 +
+                            2.0 * f.D1l * f.Du1 * f.D1r * f.Dd1 + 2.0 * f.D2l * f.Dd1 * f.D2r * f.Dd2);
+    }
+    char key[96];
+    snprintf(key, sizeof(key), "step4 f32 %d %d %d %d (%d)", f.cT, f.cB, f.cT2, f.cB2, n0 + n1);
+    return timed(0, [&] { return env4_f32(f, o, rev, st); }, key, flops);
+  }
+
   // Fused four-line step (four products in one tensor-core kernel).
+  bool spans4(const Env4Fused& f) {
+    const long long b1 = C - 1;
+    return span(f.E, b1 * f.bsE + (f.cT - 1) * f.sEa + (f.D1l - 1) * f.sEl1 + (f.D2l - 1) * f.sEl2 + (f.cB - 1) * f.sEb, 4,
+                "fused4 E") &&
+           span(f.T, b1 * f.bsT + (f.cT - 1) * f.sTa + (f.Du1 - 1) * f.sTu + (f.cT2 - 1) * f.sTa2, 4, "fused4 T") &&
+           span(f.A1, f.ss1 + (f.D1l - 1) * f.s1l + (f.Du1 - 1) * f.s1u + (f.D1r - 1) * f.s1r + (f.Dd1 - 1) * f.s1d, 4,
+                "fused4 a1") &&
+           span(f.A2, f.ss2 + (f.D2l - 1) * f.s2l + (f.Dd1 - 1) * f.s2u + (f.D2r - 1) * f.s2r + (f.Dd2 - 1) * f.s2d, 4,
+                "fused4 a2") &&
+           span(f.B, b1 * f.bsB + (f.cB - 1) * f.sBb + (f.Dd2 - 1) * f.sBd + (f.cB2 - 1) * f.sBb2, 4, "fused4 B") &&
+           span(f.out, b1 * f.bsO + (f.cT2 - 1) * f.sOa2 + (f.D1r - 1) * f.sOr1 + (f.D2r - 1) * f.sOr2 + (f.cB2 - 1) * f.sOb2,
+                4, "fused4 out") &&
+           span(f.sel1, b1 * f.sel_stride, 1, "fused4 spin 1") && span(f.sel2, b1 * f.sel_stride, 1, "fused4 spin 2");
+  }
   cudaError_t fused4(Env4Fused f) {
     f.batch = C;
     f.wait_cycles = wait_budget;
-    const long long b1 = C - 1;
-    if (!span(f.E, b1 * f.bsE + (f.cT - 1) * f.sEa + (f.D1l - 1) * f.sEl1 + (f.D2l - 1) * f.sEl2 + (f.cB - 1) * f.sEb,
-              4, "fused4 E") ||
-        !span(f.T, b1 * f.bsT + (f.cT - 1) * f.sTa + (f.Du1 - 1) * f.sTu + (f.cT2 - 1) * f.sTa2, 4, "fused4 T") ||
-        !span(f.A1, f.ss1 + (f.D1l - 1) * f.s1l + (f.Du1 - 1) * f.s1u + (f.D1r - 1) * f.s1r + (f.Dd1 - 1) * f.s1d, 4,
-              "fused4 a1") ||
-        !span(f.A2, f.ss2 + (f.D2l - 1) * f.s2l + (f.Dd1 - 1) * f.s2u + (f.D2r - 1) * f.s2r + (f.Dd2 - 1) * f.s2d, 4,
-              "fused4 a2") ||
-        !span(f.B, b1 * f.bsB + (f.cB - 1) * f.sBb + (f.Dd2 - 1) * f.sBd + (f.cB2 - 1) * f.sBb2, 4, "fused4 B") ||
-        !span(f.out, b1 * f.bsO + (f.cT2 - 1) * f.sOa2 + (f.D1r - 1) * f.sOr1 + (f.D2r - 1) * f.sOr2 +
-                         (f.cB2 - 1) * f.sOb2, 4, "fused4 out") ||
-        !span(f.sel1, b1 * f.sel_stride, 1, "fused4 spin 1") || !span(f.sel2, b1 * f.sel_stride, 1, "fused4 spin 2"))
-      return cudaErrorInvalidValue;
+    if (!spans4(f)) return cudaErrorInvalidValue;
     ++launches;
     const double nb = C;
     const double flops = 2.0 * nb *
@@ -690,6 +749,8 @@ struct pepsvmc_ctx {
                     long long bsO) {
     if (fused_ok(cT, cB, cT2, cB2, a))
       return fused3(fused_left(E, bsE, cT, cB, T, bsT, cT2, a, flip, B, bsB, cB2, out, bsO));
+    const Env3Fused f = fused_left(E, bsE, cT, cB, T, bsT, cT2, a, flip, B, bsB, cB2, out, bsO);
+    if (f32_ok(f)) return step3_f32(f, nullptr, false);
     GemmDesc g[3];
     env3_left_descs(g, Env3Dims{cT, cB, cT2, cB2, a.Dl, a.Dr, a.Du, a.Dd}, E, bsE, T, bsT, a.lurd, a.size,
                     (sel_base ? sel_base : spins) + a.spin, (long long)Ly * Lx, flip, B, bsB, out, bsO, tmp1, tmp2, SI);
@@ -715,6 +776,11 @@ struct pepsvmc_ctx {
     }
     env3_left_descs(g, d, E, bsE, T, bsT, a.lurd, a.size, (sel_base ? sel_base : spins) + a.spin, (long long)Ly * Lx, 0, B, bsB, out0, bsO,
                     tmp1, tmp2, SI);
+    const Env3Fused f = fused_left(E, bsE, cT, cB, T, bsT, cT2, a, 0, B, bsB, cB2, out0, bsO);
+    if (f32_ok(f)) {
+      PV_CUDA(step3_f32(f, out1, false));
+      return keep_et ? gemm(g[0]) : cudaSuccess;
+    }
     for (int i = 0; i < 3; ++i) PV_CUDA(gemm(g[i]));
     if (!out1) return cudaSuccess;
     env3_left_descs(g, d, E, bsE, T, bsT, a.lurd, a.size, (sel_base ? sel_base : spins) + a.spin, (long long)Ly * Lx, 1, B, bsB, out1, bsO,
@@ -729,6 +795,8 @@ struct pepsvmc_ctx {
                      long long bsO) {
     if (fused_ok(cT2, cB2, cT, cB, a))
       return fused3(fused_right(E, bsE, cT2, cB2, T, bsT, cT, a, flip, B, bsB, cB, out, bsO));
+    const Env3Fused f = fused_right(E, bsE, cT2, cB2, T, bsT, cT, a, flip, B, bsB, cB, out, bsO);
+    if (f32_ok(f)) return step3_f32(f, nullptr, true);
     PV_CUDA(right3_head(E, bsE, cT2, cB2, T, bsT, cT, a, flip));
     return right3_tail(a, cT, cB2, B, bsB, cB, out, bsO);
   }
@@ -761,6 +829,8 @@ struct pepsvmc_ctx {
       PV_CUDA(fused3(fused_right(E, bsE, cT2, cB2, T, bsT, cT, a, 0, B, bsB, cB, out0, bsO)));
       return fused3(fused_right(E, bsE, cT2, cB2, T, bsT, cT, a, 1, B, bsB, cB, out1, bsO));
     }
+    const Env3Fused f = fused_right(E, bsE, cT2, cB2, T, bsT, cT, a, 0, B, bsB, cB, out0, bsO);
+    if (f32_ok(f)) return step3_f32(f, out1, true);
     PV_CUDA(right3_head(E, bsE, cT2, cB2, T, bsT, cT, a, 0));
     PV_CUDA(right3_tail(a, cT, cB2, B, bsB, cB, out0, bsO));
     PV_CUDA(right3_head(E, bsE, cT2, cB2, T, bsT, cT, a, 1, false));
@@ -868,6 +938,9 @@ struct pepsvmc_ctx {
                     float* out, long long bsO) {
     if (four_bmajor())
       return fused4(fused4_left(E, bsE, cT, cB, T, bsT, cT2, a1, f1, a2, f2, B, bsB, cB2, out, bsO));
+    const Env4Fused f = fused4_left(E, bsE, cT, cB, T, bsT, cT2, a1, f1, a2, f2, B, bsB, cB2, out, bsO);
+    const Env4Outs o{{out}};
+    if (f32_fused() && env4_f32_fits(f, o)) return step4_f32(f, o, false);
     PV_CUDA(left4_x(E, bsE, cT, cB, T, bsT, cT2, a1, a2, tmp1));
     PV_CUDA(left4_y(tmp1, cB, cT2, a1, f1, a2, tmp2));
     return left4_zw(tmp2, cB, cT2, a1, a2, f2, B, bsB, cB2, out, bsO, tmp1);
@@ -923,6 +996,9 @@ struct pepsvmc_ctx {
                      float* out, long long bsO) {
     if (four_bmajor())
       return fused4(fused4_right(E, bsE, cT2, cB2, T, bsT, cT, a1, f1, a2, f2, B, bsB, cB, out, bsO));
+    const Env4Fused f = fused4_right(E, bsE, cT2, cB2, T, bsT, cT, a1, f1, a2, f2, B, bsB, cB, out, bsO);
+    const Env4Outs o{{out}};
+    if (f32_fused() && env4_f32_fits(f, o)) return step4_f32(f, o, true);
     const int D1l = a1.Dl, D1r = a1.Dr, Du1 = a1.Du, Dd1 = a1.Dd;
     const int D2l = a2.Dl, D2r = a2.Dr, Dd2 = a2.Dd;
     GemmDesc g;
@@ -1413,9 +1489,21 @@ struct pepsvmc_ctx {
       };
       // with the fused kernel every variant is one launch from Lin; otherwise the four
       // variants share X = Lin . T and Y(f1) = X . a1
+      // (and in FP32 one launch computes all variants with the intermediates in shared memory)
       const bool fz = four_bmajor();
+      float *Ptn = nullptr, *Pbn = nullptr;
+      if (cfg.J2 != 0.0 && !edge) {
+        Ptn = ptop[(m + 1) % 2];
+        Pbn = pbot[(m + 1) % 2];
+      }
+      const Env4Fused f4 = fused4_left(Lin, bsL, tb[m], bb[m], T.site(m), T.chain_stride, tb[m + 1], a1[m], 0, a2[m], 0,
+                                       B.site(m), B.chain_stride, bb[m + 1], cur, S4);
+      const Env4Outs o4{{cur, Pbn, Ptn, fl4}};
+      const bool f32 = f32_fused() && env4_f32_fits(f4, o4);
       if (fz) {
         PV_CUDA(step(Lin, bsL, 0, 0, cur));
+      } else if (f32) {
+        PV_CUDA(step4_f32(f4, o4, false));
       } else {
         PV_CUDA(left4_x(Lin, bsL, tb[m], bb[m], T.site(m), T.chain_stride, tb[m + 1], a1[m], a2[m], tmp1));
         PV_CUDA(left4_y(tmp1, bb[m], tb[m + 1], a1[m], 0, a2[m], tmp3));
@@ -1423,13 +1511,10 @@ struct pepsvmc_ctx {
         PV_CUDA(from_y(tmp3, 0, cur));
       }
       PV_CUDA(dot(cur, S4, Rin, bsR, n, den));
-      PV_CUDA(fz ? step(Lin, bsL, 1, 1, fl4) : from_y(tmp4, 1, fl4));
+      if (!f32) PV_CUDA(fz ? step(Lin, bsL, 1, 1, fl4) : from_y(tmp4, 1, fl4));
       PV_CUDA(ratio(fl4, S4, Rin, bsR, n, a1[m].spin, a2[m].spin, 0.5 * cfg.J1, (long long)Ly * Lx + k * Lx + m));
-      float *Ptn = nullptr, *Pbn = nullptr;
       if (cfg.J2 != 0.0) {
-        if (!edge) {
-          Ptn = ptop[(m + 1) % 2];
-          Pbn = pbot[(m + 1) % 2];
+        if (!edge && !f32) {
           PV_CUDA(fz ? step(Lin, bsL, 1, 0, Ptn) : from_y(tmp4, 0, Ptn));
           PV_CUDA(fz ? step(Lin, bsL, 0, 1, Pbn) : from_y(tmp3, 1, Pbn));
         }
@@ -1981,6 +2066,18 @@ int pepsvmc_env3_left(pepsvmc_ctx* x, const float* E, const float* T, const floa
     cudaError_t e = x->fused3(f, n_chains, true);
     return e == cudaSuccess ? PEPSVMC_OK : x->fail_cuda(e);
   }
+  if (x->f32_fused()) {
+    Env3Fused f = x->fused_left(E, (long long)cT * Dl * cB, cT, cB, T, (long long)cT * Du * cT2, cT2, op, 0, B,
+                                (long long)cB * Dd * cB2, cB2, out, (long long)cT2 * Dr * cB2);
+    f.sel = spins;
+    f.sel_stride = 1;
+    const long long no = n_chains * f.bsO;
+    if (env3_f32_fits(f) && !overlaps(out, no, E, n_chains * f.bsE) && !overlaps(out, no, T, n_chains * f.bsT) &&
+        !overlaps(out, no, A, 2 * f.ssA)) {
+      cudaError_t e = x->step3_f32(f, nullptr, false, n_chains, true);
+      return e == cudaSuccess ? PEPSVMC_OK : x->fail_cuda(e);
+    }
+  }
   GemmDesc g[3];
   env3_left_descs(g, d, E, (long long)cT * Dl * cB, T, (long long)cT * Du * cT2, A, (long long)Dl * Dr * Du * Dd,
                   spins, 1, 0, B, (long long)cB * Dd * cB2, out, (long long)cT2 * Dr * cB2, x->tmp1, x->tmp2, x->SI);
@@ -2012,31 +2109,39 @@ int pepsvmc_env4_left(pepsvmc_ctx* x, const float* E, const float* T, const floa
   Env4Fused f;
   f.cT = cT; f.cB = cB; f.cT2 = cT2; f.cB2 = cB2;
   f.D1l = D1l; f.D1r = D1r; f.Du1 = Du1; f.Dd1 = Dd1; f.D2l = D2l; f.D2r = D2r; f.Dd2 = Dd2;
+  f.batch = n_chains;
+  f.wait_cycles = x->wait_budget;
+  f.E = E; f.bsE = (long long)cT * D1l * D2l * cB;
+  if (bmajor) {
+    f.sEb = (long long)cT * D1l * D2l; f.sEa = (long long)D1l * D2l; f.sEl1 = D2l; f.sEl2 = 1;
+  } else {
+    f.sEa = (long long)D1l * D2l * cB; f.sEl1 = (long long)D2l * cB; f.sEl2 = cB; f.sEb = 1;
+  }
+  f.T = T; f.bsT = (long long)cT * Du1 * cT2; f.sTa = (long long)Du1 * cT2; f.sTu = cT2; f.sTa2 = 1;
+  f.A1 = A1; f.ss1 = s1; f.s1l = (long long)Du1 * D1r * Dd1; f.s1u = (long long)D1r * Dd1; f.s1r = Dd1; f.s1d = 1;
+  f.A2 = A2; f.ss2 = s2; f.s2l = (long long)Dd1 * D2r * Dd2; f.s2u = (long long)D2r * Dd2; f.s2r = Dd2; f.s2d = 1;
+  f.sel1 = spins1; f.sel2 = spins2; f.sel_stride = 1;
+  f.B = B; f.bsB = (long long)cB * Dd2 * cB2; f.sBb = (long long)Dd2 * cB2; f.sBd = cB2; f.sBb2 = 1;
+  f.out = out; f.bsO = (long long)cT2 * D1r * D2r * cB2;
+  if (bmajor) {
+    f.sOb2 = (long long)cT2 * D1r * D2r; f.sOa2 = (long long)D1r * D2r; f.sOr1 = D2r; f.sOr2 = 1;
+  } else {
+    f.sOa2 = (long long)D1r * D2r * cB2; f.sOr1 = (long long)D2r * cB2; f.sOr2 = cB2; f.sOb2 = 1;
+  }
   if (x->fused4_ok(f)) {
-    f.batch = n_chains;
-    f.wait_cycles = x->wait_budget;
-    f.E = E; f.bsE = (long long)cT * D1l * D2l * cB;
-    if (bmajor) {
-      f.sEb = (long long)cT * D1l * D2l; f.sEa = (long long)D1l * D2l; f.sEl1 = D2l; f.sEl2 = 1;
-    } else {
-      f.sEa = (long long)D1l * D2l * cB; f.sEl1 = (long long)D2l * cB; f.sEl2 = cB; f.sEb = 1;
-    }
-    f.T = T; f.bsT = (long long)cT * Du1 * cT2; f.sTa = (long long)Du1 * cT2; f.sTu = cT2; f.sTa2 = 1;
-    f.A1 = A1; f.ss1 = s1; f.s1l = (long long)Du1 * D1r * Dd1; f.s1u = (long long)D1r * Dd1; f.s1r = Dd1; f.s1d = 1;
-    f.A2 = A2; f.ss2 = s2; f.s2l = (long long)Dd1 * D2r * Dd2; f.s2u = (long long)D2r * Dd2; f.s2r = Dd2; f.s2d = 1;
-    f.sel1 = spins1; f.sel2 = spins2; f.sel_stride = 1;
-    f.B = B; f.bsB = (long long)cB * Dd2 * cB2; f.sBb = (long long)Dd2 * cB2; f.sBd = cB2; f.sBb2 = 1;
-    f.out = out; f.bsO = (long long)cT2 * D1r * D2r * cB2;
-    if (bmajor) {
-      f.sOb2 = (long long)cT2 * D1r * D2r; f.sOa2 = (long long)D1r * D2r; f.sOr1 = D2r; f.sOr2 = 1;
-    } else {
-      f.sOa2 = (long long)D1r * D2r * cB2; f.sOr1 = (long long)D2r * cB2; f.sOr2 = cB2; f.sOb2 = 1;
-    }
     ++x->launches;
     cudaError_t e = env4_fused(f, x->tc_mode() == 3, x->status, x->st);
     return e == cudaSuccess ? PEPSVMC_OK : x->fail_cuda(e);
   }
   if (bmajor) return x->fail(PEPSVMC_EINVAL, "env4_left: the b-major layout needs the fused kernel");
+  const Env4Outs outs{{out}};
+  const long long no = n_chains * f.bsO;
+  if (x->f32_fused() && env4_f32_fits(f, outs) && !overlaps(out, no, E, n_chains * f.bsE) &&
+      !overlaps(out, no, T, n_chains * f.bsT) && !overlaps(out, no, A1, 2 * s1) && !overlaps(out, no, A2, 2 * s2)) {
+    ++x->launches;
+    cudaError_t e = env4_f32(f, outs, false, x->st);
+    return e == cudaSuccess ? PEPSVMC_OK : x->fail_cuda(e);
+  }
   // four separate products, as left4_x / left4_y / left4_zw with the caller's spins
   GemmDesc g[4];
   float* t1 = x->tmp1;

@@ -1,0 +1,317 @@
+// Column steps in FP32 on the CUDA cores with every intermediate in shared memory (the
+// three- and four-line steps of App. C in the default precision).
+//
+// One CTA takes one chain and one tile of 8 values of the outgoing top bond a', and runs the
+// step's products one after the other.  All of them have one form: for every k in ascending
+// order, one fused multiply-add per output, rows (i, a') by columns c,
+//   S1  X(l,u | b,a')     = sum_a     T(a,u,a') E(a,l,b)          i = u,  c = (l,b)
+//   S2  Y(b,d | r,a')     = sum_(l,u) X A_s(l,u,r,d)              i = b,  c = (r,d)
+//   S3  O(a',r,b')        = sum_(b,d) Y B(b,d,b')                 i = r,  c = b'
+// (four lines: one more product between S2 and S3), which is the sum, in the same order, that
+// the separate products (contract_f32.cu) form, so results have the same bits.  a' stays the
+// fastest index of every intermediate: a thread holds 8 (or 4) values of a' by 4 (or 2)
+// columns and reads both operands as 16-byte words.
+//
+// Bound: FP32 arithmetic.  The separate products wrote and read every intermediate through
+// global memory, 4 bytes per 32-byte sector where the next product wanted another order, and
+// waited for their loads at every 16 values of k.  Measured (separate -> fused): three-line
+// step Dc 24, D 6, 2048 chains 909 -> 350 us (20 TFLOP/s), Dc 16, D 4, 1024 chains 80 -> 27 us,
+// Dc 32, D 8, 512 chains 578 -> 322 us, 64 chains of Dc 16, D 4 28 -> 11 us; four-line step
+// Dc 16, D 4, 1024 chains 385 -> 101 us.  Steps whose intermediates exceed a CTA's shared
+// memory keep the separate products.
+#include "fused_f32.cuh"
+
+namespace pv {
+namespace {
+
+constexpr int kTA = 8;        // a' per CTA
+constexpr int kMaxSmem = 227 * 1024 - 1024;
+
+// One product of the chain.  Operand P (rows): element (k, i, j) at p + k*ldp + i*8 + j; operand
+// Q (columns): element (k, c) at q + k*ldq + c (ldq and c padded to 4).  Output (i, c, j) at
+// o + (i / ni2)*si1 + (i % ni2)*si2 + (c / nc2)*sc1 + (c % nc2)*sc2 + j*sj.
+struct Product {
+  int K, ni, nc;
+  int ldp, ldq;
+  int ni2, si1, si2, nc2, sc1, sc2;
+};
+
+// TJ values of a' by TC columns per thread; tasks run c fastest, then (TJ = 4) the half of a'.
+template <int TJ, int TC, bool GLOBAL>
+__device__ __forceinline__ void product(const Product& g, const float* __restrict__ p, const float* __restrict__ q,
+                                        float* o, int sj, int nj) {
+  constexpr int H = kTA / TJ;
+  const int ncg = (g.nc + TC - 1) / TC, tasks = g.ni * H * ncg;
+  for (int t = threadIdx.x; t < tasks; t += blockDim.x) {
+    const int cg = t % ncg, ih = t / ncg, i = ih / H, j0 = (ih % H) * TJ, c0 = cg * TC;
+    const float* pp = p + i * kTA + j0;
+    const float* qq = q + c0;
+    float2 acc[TC][TJ / 2];
+#pragma unroll
+    for (int c = 0; c < TC; ++c)
+#pragma unroll
+      for (int j = 0; j < TJ / 2; ++j) acc[c][j] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int k = 0; k < g.K; ++k) {
+      float2 a[TJ / 2];
+      float b[TC];
+#pragma unroll
+      for (int j = 0; j < TJ; j += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(pp + j);
+        a[j / 2] = make_float2(v.x, v.y);
+        a[j / 2 + 1] = make_float2(v.z, v.w);
+      }
+      if constexpr (TC == 4) {
+        const float4 v = *reinterpret_cast<const float4*>(qq);
+        b[0] = v.x; b[1] = v.y; b[2] = v.z; b[3] = v.w;
+      } else {
+        const float2 v = *reinterpret_cast<const float2*>(qq);
+        b[0] = v.x; b[1] = v.y;
+      }
+#pragma unroll
+      for (int c = 0; c < TC; ++c)
+#pragma unroll
+        for (int j = 0; j < TJ / 2; ++j) acc[c][j] = __ffma2_rn(a[j], make_float2(b[c], b[c]), acc[c][j]);
+      pp += g.ldp;
+      qq += g.ldq;
+    }
+    const int oi = (i / g.ni2) * g.si1 + (i % g.ni2) * g.si2;
+#pragma unroll
+    for (int c = 0; c < TC; ++c) {
+      if (c0 + c >= g.nc) break;
+      float* d = o + oi + ((c0 + c) / g.nc2) * g.sc1 + ((c0 + c) % g.nc2) * g.sc2 + j0 * sj;
+      if constexpr (!GLOBAL) {
+#pragma unroll
+        for (int j = 0; j < TJ; j += 4)
+          *reinterpret_cast<float4*>(d + j) =
+              make_float4(acc[c][j / 2].x, acc[c][j / 2].y, acc[c][j / 2 + 1].x, acc[c][j / 2 + 1].y);
+      } else {
+#pragma unroll
+        for (int j = 0; j < TJ; ++j)
+          if (j0 + j < nj) d[j * sj] = (j & 1) ? acc[c][j / 2].y : acc[c][j / 2].x;
+      }
+    }
+  }
+}
+// The widest tile that still gives every thread something to do.
+template <bool GLOBAL>
+__device__ __forceinline__ void run(const Product& g, const float* p, const float* q, float* o, int sj = 1, int nj = kTA) {
+  const int cols4 = (g.nc + 3) / 4;
+  if (2 * g.ni * cols4 > (int)blockDim.x) product<8, 4, GLOBAL>(g, p, q, o, sj, nj);
+  else product<4, 2, GLOBAL>(g, p, q, o, sj, nj);
+}
+
+// dst[k*ld + c] for k < n0 * n1 (n0 outer), c < nc, c = (c / nc2, c % nc2), zero up to ld.
+__device__ __forceinline__ void load_cols(float* dst, int ld, const float* src, int n0, int s0, int n1, int s1, int nc,
+                                          int nc2, int sc1, int sc2) {
+  // a dense block in the same order: 16-byte copies
+  if (ld == nc && sc2 == 1 && (nc == nc2 || sc1 == nc2) && (n1 == 1 || s1 == nc) && s0 == n1 * nc && (nc & 3) == 0 &&
+      (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+    const int n = n0 * n1 * nc / 4;
+    for (int e = threadIdx.x; e < n; e += blockDim.x)
+      reinterpret_cast<float4*>(dst)[e] = reinterpret_cast<const float4*>(src)[e];
+    return;
+  }
+  const int n = n0 * n1 * ld;
+  for (int e = threadIdx.x; e < n; e += blockDim.x) {
+    const int c = e % ld, k = e / ld;
+    dst[e] = c < nc ? src[(k / n1) * s0 + (k % n1) * s1 + (c / nc2) * sc1 + (c % nc2) * sc2] : 0.f;
+  }
+}
+// T tile: dst[(a*Du + u)*8 + j], zero beyond the bond.
+__device__ __forceinline__ void load_top(float* dst, const float* T, int cT, int Du, int sTa, int sTu, int sTa2, int nj) {
+  const int n = cT * Du * kTA;
+  if (sTa2 == 1 || sTa != 1) {
+    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+      const int j = e % kTA, au = e / kTA;
+      dst[e] = j < nj ? T[(au / Du) * sTa + (au % Du) * sTu + j * sTa2] : 0.f;
+    }
+  } else {  // a contiguous (mirrored view): lanes along a
+    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+      const int a = e % cT, ju = e / cT, j = ju / Du, u = ju % Du;
+      dst[(a * Du + u) * kTA + j] = j < nj ? T[a + u * sTu + j * sTa2] : 0.f;
+    }
+  }
+}
+__host__ __device__ inline int pad4(int n) { return (n + 3) & ~3; }
+
+__device__ __forceinline__ int slot_of(const int8_t* sel, long long stride, int flip, int c) {
+  return sel ? ((sel[c * stride] < 0) ? 1 : 0) ^ flip : 0;
+}
+
+// Floats of shared memory: E, T, A, B, X, Y.
+__host__ __device__ inline void layout3(const Env3Fused& a, int off[7]) {
+  off[0] = 0;
+  off[1] = off[0] + a.cT * pad4(a.Dl * a.cB);
+  off[2] = off[1] + a.cT * a.Du * kTA;
+  off[3] = off[2] + a.Dl * a.Du * pad4(a.Dr * a.Dd);
+  off[4] = off[3] + a.cB * a.Dd * pad4(a.cB2);
+  off[5] = off[4] + a.Dl * a.Du * a.cB * kTA;
+  off[6] = off[5] + a.cB * a.Dd * a.Dr * kTA;
+}
+
+__global__ void __launch_bounds__(256) env3_f32_kernel(const Env3Fused a, float* out1, bool rev) {
+  extern __shared__ __align__(16) float sf[];
+  int off[7];
+  layout3(a, off);
+  float *E = sf + off[0], *T = sf + off[1], *A = sf + off[2], *B = sf + off[3], *X = sf + off[4], *Y = sf + off[5];
+  const int n_at = (a.cT2 + kTA - 1) / kTA, c = blockIdx.x / n_at, a0 = (blockIdx.x % n_at) * kTA;
+  const int nj = min(kTA, a.cT2 - a0);
+  const int slot = slot_of(a.sel, a.sel_stride, a.sel_xor, c);
+  const int ldE = pad4(a.Dl * a.cB), ldA = pad4(a.Dr * a.Dd), ldB = pad4(a.cB2);
+  const int sAl = (int)a.sAl, sAu = (int)a.sAu, sAr = (int)a.sAr, sAd = (int)a.sAd;
+  auto load_site = [&](int s) {
+    const float* src = a.A + s * a.ssA;
+    if (rev) load_cols(A, ldA, src, a.Du, sAu, a.Dl, sAl, a.Dr * a.Dd, a.Dd, sAr, sAd);
+    else load_cols(A, ldA, src, a.Dl, sAl, a.Du, sAu, a.Dr * a.Dd, a.Dd, sAr, sAd);
+  };
+  load_cols(E, ldE, a.E + c * a.bsE, a.cT, (int)a.sEa, 1, 0, a.Dl * a.cB, a.cB, (int)a.sEl, (int)a.sEb);
+  load_top(T, a.T + c * a.bsT + a0 * a.sTa2, a.cT, a.Du, (int)a.sTa, (int)a.sTu, (int)a.sTa2, nj);
+  load_site(slot);
+  if (rev) load_cols(B, ldB, a.B + c * a.bsB, a.Dd, (int)a.sBd, a.cB, (int)a.sBb, a.cB2, a.cB2, 0, (int)a.sBb2);
+  else load_cols(B, ldB, a.B + c * a.bsB, a.cB, (int)a.sBb, a.Dd, (int)a.sBd, a.cB2, a.cB2, 0, (int)a.sBb2);
+  __syncthreads();
+  const int ldX = a.cB * kTA, ldY = a.Dr * kTA;
+  const int xl = rev ? ldX : a.Du * ldX, xu = rev ? a.Dl * ldX : ldX;
+  const int yb = rev ? ldY : a.Dd * ldY, yd = rev ? a.cB * ldY : ldY;
+  run<false>(Product{a.cT, a.Du, a.Dl * a.cB, a.Du * kTA, ldE, a.Du, 0, xu, a.cB, xl, kTA}, T, E, X);
+  __syncthreads();
+  const Product s2{a.Dl * a.Du, a.cB, a.Dr * a.Dd, ldX, ldA, a.cB, 0, yb, a.Dd, kTA, yd};
+  const Product s3{a.cB * a.Dd, a.Dr, a.cB2, ldY, ldB, a.Dr, 0, (int)a.sOr, a.cB2, 0, (int)a.sOb2};
+  for (int v = 0; v < 2; ++v) {
+    float* O = v ? out1 : a.out;
+    if (!O) break;
+    if (v) {  // the other slot of the site, X shared
+      load_site(slot ^ 1);
+      __syncthreads();
+    }
+    run<false>(s2, X, A, Y);
+    __syncthreads();
+    run<true>(s3, Y, B, O + c * a.bsO + a0 * a.sOa2, (int)a.sOa2, nj);
+    if (v == 0 && out1) __syncthreads();
+  }
+}
+
+// Floats of shared memory: E, T, A1, A2, B, X, Y, Z; with one variant Z takes X's place.
+__host__ __device__ inline void layout4(const Env4Fused& a, bool several, int off[9]) {
+  const int x = a.D1l * a.Du1 * a.D2l * a.cB * kTA, z = a.cB * a.Dd2 * a.D1r * a.D2r * kTA;
+  off[0] = 0;
+  off[1] = off[0] + a.cT * pad4(a.D1l * a.D2l * a.cB);
+  off[2] = off[1] + a.cT * a.Du1 * kTA;
+  off[3] = off[2] + a.D1l * a.Du1 * pad4(a.D1r * a.Dd1);
+  off[4] = off[3] + a.D2l * a.Dd1 * pad4(a.D2r * a.Dd2);
+  off[5] = off[4] + a.cB * a.Dd2 * pad4(a.cB2);
+  off[6] = off[5] + (several || x > z ? x : z);
+  off[7] = off[6] + a.D2l * a.Dd1 * a.cB * a.D1r * kTA;
+  off[8] = off[7] + (several ? z : 0);
+}
+
+__global__ void __launch_bounds__(256) env4_f32_kernel(const Env4Fused a, const Env4Outs outs, bool several, bool rev) {
+  extern __shared__ __align__(16) float sf[];
+  int off[9];
+  layout4(a, several, off);
+  float *E = sf + off[0], *T = sf + off[1], *A1 = sf + off[2], *A2 = sf + off[3], *B = sf + off[4], *X = sf + off[5],
+        *Y = sf + off[6], *Z = several ? sf + off[7] : X;
+  const int n_at = (a.cT2 + kTA - 1) / kTA, c = blockIdx.x / n_at, a0 = (blockIdx.x % n_at) * kTA;
+  const int nj = min(kTA, a.cT2 - a0);
+  const int nE = a.D1l * a.D2l * a.cB, ldE = pad4(nE), ld1 = pad4(a.D1r * a.Dd1), ld2 = pad4(a.D2r * a.Dd2),
+            ldB = pad4(a.cB2);
+  const int slot1 = slot_of(a.sel1, a.sel_stride, a.xor1, c), slot2 = slot_of(a.sel2, a.sel_stride, a.xor2, c);
+  auto load1 = [&](int s) {
+    const float* src = a.A1 + s * a.ss1;
+    if (rev) load_cols(A1, ld1, src, a.Du1, (int)a.s1u, a.D1l, (int)a.s1l, a.D1r * a.Dd1, a.Dd1, (int)a.s1r, (int)a.s1d);
+    else load_cols(A1, ld1, src, a.D1l, (int)a.s1l, a.Du1, (int)a.s1u, a.D1r * a.Dd1, a.Dd1, (int)a.s1r, (int)a.s1d);
+  };
+  auto load2 = [&](int s) {
+    const float* src = a.A2 + s * a.ss2;
+    if (rev) load_cols(A2, ld2, src, a.Dd1, (int)a.s2u, a.D2l, (int)a.s2l, a.D2r * a.Dd2, a.Dd2, (int)a.s2r, (int)a.s2d);
+    else load_cols(A2, ld2, src, a.D2l, (int)a.s2l, a.Dd1, (int)a.s2u, a.D2r * a.Dd2, a.Dd2, (int)a.s2r, (int)a.s2d);
+  };
+  // E's columns (l1, l2, b): l1 and l2 are one index of stride sEl2 (dense storage)
+  load_cols(E, ldE, a.E + c * a.bsE, a.cT, (int)a.sEa, 1, 0, nE, a.cB, (int)a.sEl2, (int)a.sEb);
+  load_top(T, a.T + c * a.bsT + a0 * a.sTa2, a.cT, a.Du1, (int)a.sTa, (int)a.sTu, (int)a.sTa2, nj);
+  if (rev) load_cols(B, ldB, a.B + c * a.bsB, a.Dd2, (int)a.sBd, a.cB, (int)a.sBb, a.cB2, a.cB2, 0, (int)a.sBb2);
+  else load_cols(B, ldB, a.B + c * a.bsB, a.cB, (int)a.sBb, a.Dd2, (int)a.sBd, a.cB2, a.cB2, 0, (int)a.sBb2);
+  const int n2b = a.D2l * a.cB, ldX = n2b * kTA, ldY = a.cB * a.D1r * kTA, ldZ = a.D1r * a.D2r * kTA;
+  const int xl = rev ? ldX : a.Du1 * ldX, xu = rev ? a.D1l * ldX : ldX;
+  const int yl = rev ? ldY : a.Dd1 * ldY, yd = rev ? a.D2l * ldY : ldY;
+  const int zb = rev ? ldZ : a.Dd2 * ldZ, zd = rev ? a.cB * ldZ : ldZ;
+  bool fresh = true;
+  for (int f1 = 0; f1 < 2; ++f1) {
+    if (!outs.p[2 * f1] && !outs.p[2 * f1 + 1]) continue;
+    load1(slot1 ^ f1);
+    __syncthreads();
+    // X(l1,u1 | l2,b): columns (l1, (l2,b)), rows u1
+    if (fresh) {
+      run<false>(Product{a.cT, a.Du1, nE, a.Du1 * kTA, ldE, a.Du1, 0, xu, n2b, xl, kTA}, T, E, X);
+      __syncthreads();
+      fresh = false;
+    }
+    // Y(l2,d1 | b,r1): rows (l2, b), columns (r1, d1)
+    run<false>(Product{a.D1l * a.Du1, n2b, a.D1r * a.Dd1, ldX, ld1, a.cB, yl, a.D1r * kTA, a.Dd1, kTA, yd}, X, A1, Y);
+    for (int f2 = 0; f2 < 2; ++f2) {
+      float* O = outs.p[2 * f1 + f2];
+      if (!O) continue;
+      load2(slot2 ^ f2);
+      __syncthreads();
+      // Z(b,d2 | r1,r2): rows (b, r1), columns (r2, d2)
+      run<false>(Product{a.D2l * a.Dd1, a.cB * a.D1r, a.D2r * a.Dd2, ldY, ld2, a.D1r, zb, a.D2r * kTA, a.Dd2, kTA, zd}, Y, A2, Z);
+      __syncthreads();
+      // O(a',r1,r2,b'): rows (r1, r2), columns b'
+      run<true>(Product{a.cB * a.Dd2, a.D1r * a.D2r, a.cB2, ldZ, ldB, a.D2r, (int)a.sOr1, (int)a.sOr2, a.cB2, 0, (int)a.sOb2},
+                Z, B, O + c * a.bsO + a0 * a.sOa2, (int)a.sOa2, nj);
+    }
+  }
+}
+
+// Threads of a CTA: enough for the first products' tasks of 8 x 4, at most 256.
+int threads_for(int tasks) { return tasks > 128 ? 256 : tasks > 64 ? 128 : 64; }
+
+template <typename K>
+cudaError_t allow_smem(K kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+}
+
+}  // namespace
+
+bool env3_f32_fits(const Env3Fused& a) {
+  int off[7];
+  layout3(a, off);
+  return (long long)off[6] * 4 <= kMaxSmem;
+}
+
+cudaError_t env3_f32(const Env3Fused& a, float* out1, bool rev, cudaStream_t st) {
+  if (g_dry_run || a.batch <= 0) return cudaSuccess;
+  int off[7];
+  layout3(a, off);
+  static const cudaError_t allowed = allow_smem(env3_f32_kernel);
+  PV_CUDA(allowed);
+  const long long blocks = (long long)a.batch * ((a.cT2 + kTA - 1) / kTA);
+  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+  const int tasks = a.Du * ((a.Dl * a.cB + 3) / 4), tasks2 = a.cB * ((a.Dr * a.Dd + 3) / 4);
+  env3_f32_kernel<<<(unsigned)blocks, threads_for(tasks > tasks2 ? tasks : tasks2), off[6] * 4, st>>>(a, out1, rev);
+  return cudaGetLastError();
+}
+
+static bool several(const Env4Outs& o) { return (o.p[0] != nullptr) + (o.p[1] != nullptr) + (o.p[2] != nullptr) + (o.p[3] != nullptr) > 1; }
+
+bool env4_f32_fits(const Env4Fused& a, const Env4Outs& outs) {
+  int off[9];
+  layout4(a, several(outs), off);
+  return a.sEl1 == (long long)a.D2l * a.sEl2 && (long long)off[8] * 4 <= kMaxSmem;
+}
+
+cudaError_t env4_f32(const Env4Fused& a, const Env4Outs& outs, bool rev, cudaStream_t st) {
+  if (g_dry_run || a.batch <= 0) return cudaSuccess;
+  int off[9];
+  layout4(a, several(outs), off);
+  static const cudaError_t allowed = allow_smem(env4_f32_kernel);
+  PV_CUDA(allowed);
+  const long long blocks = (long long)a.batch * ((a.cT2 + kTA - 1) / kTA);
+  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+  const int tasks = a.D2l * a.cB * ((a.D1r * a.Dd1 + 3) / 4);
+  env4_f32_kernel<<<(unsigned)blocks, threads_for(tasks), off[8] * 4, st>>>(a, outs, several(outs), rev);
+  return cudaGetLastError();
+}
+
+}  // namespace pv

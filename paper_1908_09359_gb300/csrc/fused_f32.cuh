@@ -1,0 +1,23 @@
+// Column steps in FP32 on the CUDA cores, all products of a step in one kernel.
+#pragma once
+#include "fused.cuh"
+
+namespace pv {
+
+// Three-line step of every chain as Env3Fused describes it (any strides); out1 (nullable):
+// the result with the other slot of the site tensor, sharing E . T.  rev: the sums over (l, u)
+// and (b, d) run u and d slowest (as the separate products of a right step do) instead of l
+// and b.  Sums ascend in k with one fused multiply-add per term, as gemm_f32's do.
+bool env3_f32_fits(const Env3Fused& a);
+cudaError_t env3_f32(const Env3Fused& a, float* out1, bool rev, cudaStream_t st);
+
+// Four-line step; p[2 f1 + f2] (nullable): the result with the slots of the two sites flipped by
+// f1 and f2, sharing E . T and, between the two f2, the product with a1.  rev: the sums over
+// (l1, u1), (l2, d1) and (b, d2) run the second index slowest.
+struct Env4Outs {
+  float* p[4] = {};
+};
+bool env4_f32_fits(const Env4Fused& a, const Env4Outs& outs);
+cudaError_t env4_f32(const Env4Fused& a, const Env4Outs& outs, bool rev, cudaStream_t st);
+
+}  // namespace pv

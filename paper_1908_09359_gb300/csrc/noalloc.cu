@@ -16,6 +16,7 @@
 // address right after a device reset or when another context is current on the device.
 
 #include "common.cuh"
+#include "fused_f32.cuh"
 #include "pepsvmc.h"
 #include "stages.cuh"
 
@@ -43,6 +44,20 @@ extern "C" int pepsvmc_env3_left_noalloc(const float* E, const float* T, const f
   if (!E || !T || !A || !B || !out || n_chains < 1 || !env3_dims_ok(d)) return PEPSVMC_EINVAL;
   const long long per_chain = env3_scratch(d);
   if (per_chain > PEPSVMC_NOALLOC_SCRATCH_FLOATS / 2 / n_chains) return PEPSVMC_EINVAL;  // does not fit
+  Env3Fused f;  // all intermediates in shared memory where they fit
+  f.cT = cT; f.cB = cB; f.cT2 = cT2; f.cB2 = cB2; f.Dl = Dl; f.Dr = Dr; f.Du = Du; f.Dd = Dd;
+  f.batch = n_chains;
+  f.E = E; f.bsE = (long long)cT * Dl * cB; f.sEa = (long long)Dl * cB; f.sEl = cB; f.sEb = 1;
+  f.T = T; f.bsT = (long long)cT * Du * cT2; f.sTa = (long long)Du * cT2; f.sTu = cT2; f.sTa2 = 1;
+  f.A = A; f.ssA = (long long)Dl * Dr * Du * Dd;
+  f.sAl = (long long)Du * Dr * Dd; f.sAu = (long long)Dr * Dd; f.sAr = Dd; f.sAd = 1;
+  f.sel = spins; f.sel_stride = 1;
+  f.B = B; f.bsB = (long long)cB * Dd * cB2; f.sBb = (long long)Dd * cB2; f.sBd = cB2; f.sBb2 = 1;
+  f.out = out; f.bsO = (long long)cT2 * Dr * cB2; f.sOa2 = (long long)Dr * cB2; f.sOr = cB2; f.sOb2 = 1;
+  const long long no = n_chains * f.bsO;
+  if (env3_f32_fits(f) && !overlaps(out, no, E, n_chains * f.bsE) && !overlaps(out, no, T, n_chains * f.bsT) &&
+      !overlaps(out, no, A, 2 * f.ssA))
+    return env3_f32(f, nullptr, false, (cudaStream_t)stream) == cudaSuccess ? PEPSVMC_OK : PEPSVMC_ECUDA;
   float* scratch = nullptr;
   const int rc = scratch_on_current_device(&scratch);
   if (rc != PEPSVMC_OK) return rc;

@@ -49,6 +49,11 @@ inline long long env3_scratch(const Env3Dims& d) {
   return a > b ? a : b;
 }
 
+// Whether n floats at p and m floats at q share memory.  The separate products read E, T and A
+// before they write the result, the one-kernel steps do not: a caller whose result lies over
+// one of those gets the separate products.
+inline bool overlaps(const float* p, long long n, const float* q, long long m) { return p < q + m && q < p + n; }
+
 inline bool env3_dims_ok(const Env3Dims& d) {
   return d.cT > 0 && d.cB > 0 && d.cT2 > 0 && d.cB2 > 0 && d.Dl > 0 && d.Dr > 0 && d.Du > 0 && d.Dd > 0;
 }
