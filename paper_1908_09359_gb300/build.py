@@ -18,7 +18,7 @@ OUT = os.path.join(HERE, "_build")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(OUT, "libpepsvmc.so")
 
-SOURCES = ["contract_f32.cu", "contract_tc.cu", "fused_env3.cu", "fused_env3_tiles.cu", "fused_env4.cu", "fused_f32.cu", "qr.cu", "kernels.cu", "engine.cu", "noalloc.cu",
+SOURCES = ["contract_f32.cu", "contract_tc.cu", "fused_env3.cu", "fused_env3_tiles.cu", "fused_env4.cu", "fused_env4_pipe.cu", "fused_f32.cu", "qr.cu", "kernels.cu", "engine.cu", "noalloc.cu",
            "simple_update.cu",
            "proposal.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

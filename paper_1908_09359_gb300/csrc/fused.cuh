@@ -90,6 +90,12 @@ inline bool env4_fused_fits(const Env4Fused& f) {
 
 cudaError_t env4_fused(const Env4Fused& a, bool split, unsigned* status, cudaStream_t st);
 
+// The pipeline of full bonds (fused_env4_pipe.cu): whether it takes this step (the
+// launch plan is then in `plan`), and the launch; env4_fused chooses.
+constexpr size_t kEnv4PlanBytes = 1024;
+bool env4_pipe_fits(const Env4Fused& a, void* plan);
+cudaError_t env4_pipe(const void* plan, bool split, unsigned* status, cudaStream_t st);
+
 }  // namespace pv
 
 namespace pv {

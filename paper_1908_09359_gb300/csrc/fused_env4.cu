@@ -19,7 +19,7 @@
 // plus A_lo x B_hi, and the epilogue adds the two column halves (the lo copy of each B
 // tile directly follows its hi copy with the same row-group stride).  The E and B slices
 // of the next b tile are fetched into registers while the current tile computes.  Bonds
-// below the maxima are zero-padded on chip.  Shared memory 93 KB and 256 tensor-memory
+// below the maxima are zero-padded on chip.  (Full bonds run in fused_env4_pipe.cu.)  Shared memory 93 KB and 256 tensor-memory
 // columns per CTA: two CTAs share an SM, so one CTA's epilogues overlap the other's
 // products.
 #include "fused.cuh"
@@ -356,6 +356,11 @@ cudaError_t launch(const Env4Fused& a, unsigned* status, cudaStream_t st) {
 cudaError_t env4_fused(const Env4Fused& a, bool split, unsigned* status, cudaStream_t st) {
   if (g_dry_run || a.batch <= 0) return cudaSuccess;
   if (!env4_fused_fits(a)) return cudaErrorInvalidValue;
+  // Full bonds, b-major and dense: the pipeline, at every number of chains (61 -> 41 us at one,
+  // 566 -> 439 us at 512).  Its conversions have no bounds; smaller bonds and other orders
+  // of E's indices stay with the kernel above.
+  alignas(16) unsigned char plan[kEnv4PlanBytes];
+  if (env4_pipe_fits(a, plan)) return env4_pipe(plan, split, status, st);
   return split ? launch<true>(a, status, st) : launch<false>(a, status, st);
 }
 

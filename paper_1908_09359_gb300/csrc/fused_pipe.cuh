@@ -36,7 +36,7 @@ struct PipeCtl {
   unsigned* status;
   long long budget;
 };
-__device__ __noinline__ bool pipe_wait(uint32_t bar, uint32_t parity, PipeCtl* ctl) {
+static __device__ __noinline__ bool pipe_wait(uint32_t bar, uint32_t parity, PipeCtl* ctl) {
   uint32_t done;
   asm volatile(
       "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
