@@ -566,7 +566,59 @@ struct pepsvmc_ctx {
     }
     char key[96];
     snprintf(key, sizeof(key), "step3 f32 %d %d %d %d x %d %d %d %d", f.cT, f.cB, f.cT2, f.cB2, f.Dl, f.Dr, f.Du, f.Dd);
-    return timed(0, [&] { return env3_f32(f, out1, rev, st); }, key, flops);
+    return timed(0, [&] { return env3_f32(f, out1, rev, rev, Mid3(), st); }, key, flops);
+  }
+  // FP32 optimal site of the fit, Y (cV,Dd,cV2) = L . T . a . R, in one kernel: the same chain
+  // of products with one of the boundary bonds in the place of a'.  From the left (the sums
+  // and the copy in tmp2 are proj3's) that is v, from the right (proj3_right's) v2.
+  Env3Fused proj_f32(bool right, const float* Lf, long long bsL, int cT, int cV, const float* T, long long bsT, int cT2,
+                     const SiteOp& a, const float* Rf, long long bsR, int cV2, float* Y, long long bsY, Mid3& mid) const {
+    const int Dl = a.Dl, Dr = a.Dr, Du = a.Du, Dd = a.Dd;
+    Env3Fused f;
+    f.A = a.lurd; f.ssA = a.size; f.sAl = (long long)Dr * Dd; f.sAr = 1;
+    f.sel = (sel_base ? sel_base : spins) + a.spin; f.sel_stride = (long long)Ly * Lx;
+    f.Dl = Du; f.Dr = Dd;
+    f.E = T; f.bsE = bsT; f.sEl = cT2;
+    f.out = Y; f.bsO = bsY; f.sOr = cV2;
+    mid.p = tmp2; mid.bs = SI;
+    if (!right) {
+      f.cT = cT; f.cB = cT2; f.cT2 = cV; f.cB2 = cV2; f.Du = Dl; f.Dd = Dr;
+      f.sEa = (long long)Du * cT2; f.sEb = 1;
+      f.T = Lf; f.bsT = bsL; f.sTa = (long long)Dl * cV; f.sTu = cV; f.sTa2 = 1;
+      f.sAu = (long long)Du * Dr * Dd; f.sAd = Dd;
+      f.B = Rf; f.bsB = bsR; f.sBb = (long long)Dr * cV2; f.sBd = cV2; f.sBb2 = 1;
+      f.sOa2 = (long long)Dd * cV2; f.sOb2 = 1;
+      mid.sj = Dd * cT2 * Dr; mid.sr = cT2 * Dr; mid.sb = Dr; mid.sd = 1;
+    } else {
+      f.cT = cT2; f.cB = cT; f.cT2 = cV2; f.cB2 = cV; f.Du = Dr; f.Dd = Dl;
+      f.sEa = 1; f.sEb = (long long)Du * cT2;
+      f.T = Rf; f.bsT = bsR; f.sTa = (long long)Dr * cV2; f.sTu = cV2; f.sTa2 = 1;
+      f.sAu = Dd; f.sAd = (long long)Du * Dr * Dd;
+      f.B = Lf; f.bsB = bsL; f.sBb = (long long)Dl * cV; f.sBd = cV; f.sBb2 = 1;
+      f.sOa2 = 1; f.sOb2 = (long long)Dd * cV2;
+      mid.sj = 1; mid.sr = cV2; mid.sb = Dl * Dd * cV2; mid.sd = Dd * cV2;
+    }
+    return f;
+  }
+  cudaError_t proj_step_f32(Env3Fused f, const Mid3& mid, bool right) {
+    f.batch = C;
+    if (!spans3(f) || !chains(mid.p, mid.bs, (long long)f.cB * f.Dd * f.Dr * f.cT2, 4, "fit intermediate"))
+      return cudaErrorInvalidValue;
+    ++launches;
+    const double nb = f.batch;
+    const double flops = 2.0 * nb *
+        ((double)f.Dl * f.cB * f.Du * f.cT2 * f.cT + (double)f.cB * f.cT2 * f.Dr * f.Dd * f.Dl * f.Du +
+         (double)f.cT2 * f.Dr * f.cB2 * f.cB * f.Dd);
+    if (prof) {
+      prof_acc[0] += 1;
+      prof_acc[1] += flops;
+      prof_acc[5] += 4.0 * ((f.bsE ? nb : 1.0) * f.cT * f.Dl * f.cB + (f.bsT ? nb : 1.0) * f.cT * f.Du * f.cT2 +
+                            (f.bsB ? nb : 1.0) * f.cB * f.Dd * f.cB2 + nb * f.cT2 * f.Dr * (f.cB2 + (double)f.cB * f.Dd) +
+                            2.0 * f.Dl * f.Du * f.Dr * f.Dd);
+    }
+    char key[96];
+    snprintf(key, sizeof(key), "proj f32 %d %d %d %d x %d %d %d %d", f.cT, f.cB, f.cT2, f.cB2, f.Dl, f.Dr, f.Du, f.Dd);
+    return timed(0, [&] { return env3_f32(f, nullptr, !right, false, mid, st); }, key, flops);
   }
   // FP32 four-line step, one to four flip variants (see Env4Outs) of it in one kernel.
   cudaError_t step4_f32(Env4Fused f, const Env4Outs& o, bool rev) {
@@ -866,6 +918,9 @@ struct pepsvmc_ctx {
   // right3_tail then gives the new right environment without repeating those products.
   cudaError_t proj3_right(const float* Lf, long long bsL, int cT, int cV, const float* T, long long bsT, int cT2,
                           const SiteOp& a, const float* Rf, long long bsR, int cV2, float* Y, long long bsY) {
+    Mid3 mid;
+    const Env3Fused f = proj_f32(true, Lf, bsL, cT, cV, T, bsT, cT2, a, Rf, bsR, cV2, Y, bsY, mid);
+    if (f32_ok(f)) return proj_step_f32(f, mid, true);
     PV_CUDA(right3_head(Rf, bsR, cT2, cV2, T, bsT, cT, a, 0));
     const int Dl = a.Dl, Dd = a.Dd;
     GemmDesc q;
@@ -880,6 +935,9 @@ struct pepsvmc_ctx {
   // contracted from the left; tmp2 keeps L . T . a for left3_tail_after_proj.
   cudaError_t proj3(const float* Lf, long long bsL, int cT, int cV, const float* T, long long bsT, int cT2,
                     const SiteOp& a, const float* Rf, long long bsR, int cV2, float* Y, long long bsY) {
+    Mid3 mid;
+    const Env3Fused f = proj_f32(false, Lf, bsL, cT, cV, T, bsT, cT2, a, Rf, bsR, cV2, Y, bsY, mid);
+    if (f32_ok(f)) return proj_step_f32(f, mid, false);
     const int Dl = a.Dl, Dr = a.Dr, Du = a.Du, Dd = a.Dd;
     GemmDesc g;
     g.M = Dl * cV; g.N = Du * cT2; g.K = cT;

@@ -12,6 +12,11 @@
 // fastest index of every intermediate: a thread holds 8 (or 4) values of a' by 4 (or 2)
 // columns and reads both operands as 16-byte words.
 //
+// The optimal site of the boundary-MPS fit is the same chain of products with a boundary bond
+// in the place of a'; its middle product goes to memory as well, where the product that
+// makes the next environment reads it (fit of Dc 16, D 4, 1024 chains: 92 us in three products,
+// 41 us in one kernel, with ~6 us of event time per launch).
+//
 // Bound: FP32 arithmetic.  The separate products wrote and read every intermediate through
 // global memory, 4 bytes per 32-byte sector where the next product wanted another order, and
 // waited for their loads at every 16 values of k.  Measured (separate -> fused): three-line
@@ -37,9 +42,14 @@ struct Product {
 };
 
 // TJ values of a' by TC columns per thread; tasks run c fastest, then (TJ = 4) the half of a'.
-template <int TJ, int TC, bool GLOBAL>
+struct Copy {  // of a product's output in global memory: (i, c, j) at p + i*si + (c / nc2)*sc1 + (c % nc2)*sc2 + j*sj
+  float* p = nullptr;
+  int si = 0, sc1 = 0, sc2 = 0, sj = 0;
+  int nc2 = 1;
+};
+template <int TJ, int TC, bool GLOBAL, bool COPY>
 __device__ __forceinline__ void product(const Product& g, const float* __restrict__ p, const float* __restrict__ q,
-                                        float* o, int sj, int nj) {
+                                        float* o, int sj, int nj, const Copy& cp) {
   constexpr int H = kTA / TJ;
   const int ncg = (g.nc + TC - 1) / TC, tasks = g.ni * H * ncg;
   for (int t = threadIdx.x; t < tasks; t += blockDim.x) {
@@ -91,14 +101,40 @@ __device__ __forceinline__ void product(const Product& g, const float* __restric
           if (j0 + j < nj) d[j * sj] = (j & 1) ? acc[c][j / 2].y : acc[c][j / 2].x;
       }
     }
+    if constexpr (COPY) {
+      {
+        float* d = cp.p + i * cp.si + j0 * cp.sj;
+        const int e = c0 % cp.nc2;
+        if (TC == 4 && cp.sc2 == 1 && c0 + 3 < g.nc && e + 3 < cp.nc2 &&
+            ((reinterpret_cast<uintptr_t>(cp.p) | ((cp.si | cp.sc1 | cp.sj | e) * 4)) & 15) == 0) {
+          d += (c0 / cp.nc2) * cp.sc1 + e;
+#pragma unroll
+          for (int j = 0; j < TJ; ++j)
+            if (j0 + j < nj)
+              *reinterpret_cast<float4*>(d + j * cp.sj) =
+                  (j & 1) ? make_float4(acc[0][j / 2].y, acc[1][j / 2].y, acc[TC - 2][j / 2].y, acc[TC - 1][j / 2].y)
+                          : make_float4(acc[0][j / 2].x, acc[1][j / 2].x, acc[TC - 2][j / 2].x, acc[TC - 1][j / 2].x);
+        } else {
+#pragma unroll
+          for (int c = 0; c < TC; ++c) {
+            if (c0 + c >= g.nc) break;
+            float* f = d + ((c0 + c) / cp.nc2) * cp.sc1 + ((c0 + c) % cp.nc2) * cp.sc2;
+#pragma unroll
+            for (int j = 0; j < TJ; ++j)
+              if (j0 + j < nj) f[j * cp.sj] = (j & 1) ? acc[c][j / 2].y : acc[c][j / 2].x;
+          }
+        }
+      }
+    }
   }
 }
 // The widest tile that still gives every thread something to do.
-template <bool GLOBAL>
-__device__ __forceinline__ void run(const Product& g, const float* p, const float* q, float* o, int sj = 1, int nj = kTA) {
+template <bool GLOBAL, bool COPY = false>
+__device__ __forceinline__ void run(const Product& g, const float* p, const float* q, float* o, int sj = 1, int nj = kTA,
+                                    const Copy& cp = Copy()) {
   const int cols4 = (g.nc + 3) / 4;
-  if (2 * g.ni * cols4 > (int)blockDim.x) product<8, 4, GLOBAL>(g, p, q, o, sj, nj);
-  else product<4, 2, GLOBAL>(g, p, q, o, sj, nj);
+  if (2 * g.ni * cols4 > (int)blockDim.x) product<8, 4, GLOBAL, COPY>(g, p, q, o, sj, nj, cp);
+  else product<4, 2, GLOBAL, COPY>(g, p, q, o, sj, nj, cp);
 }
 
 // dst[k*ld + c] for k < n0 * n1 (n0 outer), c < nc, c = (c / nc2, c % nc2), zero up to ld.
@@ -113,6 +149,13 @@ __device__ __forceinline__ void load_cols(float* dst, int ld, const float* src, 
     return;
   }
   const int n = n0 * n1 * ld;
+  if (n1 == 1 && s0 == 1 && sc2 != 1) {  // k contiguous (a mirrored view): lanes along k
+    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+      const int k = e % n0, c = e / n0;
+      dst[k * ld + c] = c < nc ? src[k + (c / nc2) * sc1 + (c % nc2) * sc2] : 0.f;
+    }
+    return;
+  }
   for (int e = threadIdx.x; e < n; e += blockDim.x) {
     const int c = e % ld, k = e / ld;
     dst[e] = c < nc ? src[(k / n1) * s0 + (k % n1) * s1 + (c / nc2) * sc1 + (c % nc2) * sc2] : 0.f;
@@ -150,7 +193,8 @@ __host__ __device__ inline void layout3(const Env3Fused& a, int off[7]) {
   off[6] = off[5] + a.cB * a.Dd * a.Dr * kTA;
 }
 
-__global__ void __launch_bounds__(256) env3_f32_kernel(const Env3Fused a, float* out1, bool rev) {
+template <bool MID>
+__global__ void __launch_bounds__(256, MID ? 3 : 0) env3_f32_kernel(const Env3Fused a, float* out1, bool rev2, bool rev3, const Mid3 mid) {
   extern __shared__ __align__(16) float sf[];
   int off[7];
   layout3(a, off);
@@ -162,18 +206,18 @@ __global__ void __launch_bounds__(256) env3_f32_kernel(const Env3Fused a, float*
   const int sAl = (int)a.sAl, sAu = (int)a.sAu, sAr = (int)a.sAr, sAd = (int)a.sAd;
   auto load_site = [&](int s) {
     const float* src = a.A + s * a.ssA;
-    if (rev) load_cols(A, ldA, src, a.Du, sAu, a.Dl, sAl, a.Dr * a.Dd, a.Dd, sAr, sAd);
+    if (rev2) load_cols(A, ldA, src, a.Du, sAu, a.Dl, sAl, a.Dr * a.Dd, a.Dd, sAr, sAd);
     else load_cols(A, ldA, src, a.Dl, sAl, a.Du, sAu, a.Dr * a.Dd, a.Dd, sAr, sAd);
   };
   load_cols(E, ldE, a.E + c * a.bsE, a.cT, (int)a.sEa, 1, 0, a.Dl * a.cB, a.cB, (int)a.sEl, (int)a.sEb);
   load_top(T, a.T + c * a.bsT + a0 * a.sTa2, a.cT, a.Du, (int)a.sTa, (int)a.sTu, (int)a.sTa2, nj);
   load_site(slot);
-  if (rev) load_cols(B, ldB, a.B + c * a.bsB, a.Dd, (int)a.sBd, a.cB, (int)a.sBb, a.cB2, a.cB2, 0, (int)a.sBb2);
+  if (rev3) load_cols(B, ldB, a.B + c * a.bsB, a.Dd, (int)a.sBd, a.cB, (int)a.sBb, a.cB2, a.cB2, 0, (int)a.sBb2);
   else load_cols(B, ldB, a.B + c * a.bsB, a.cB, (int)a.sBb, a.Dd, (int)a.sBd, a.cB2, a.cB2, 0, (int)a.sBb2);
   __syncthreads();
   const int ldX = a.cB * kTA, ldY = a.Dr * kTA;
-  const int xl = rev ? ldX : a.Du * ldX, xu = rev ? a.Dl * ldX : ldX;
-  const int yb = rev ? ldY : a.Dd * ldY, yd = rev ? a.cB * ldY : ldY;
+  const int xl = rev2 ? ldX : a.Du * ldX, xu = rev2 ? a.Dl * ldX : ldX;
+  const int yb = rev3 ? ldY : a.Dd * ldY, yd = rev3 ? a.cB * ldY : ldY;
   run<false>(Product{a.cT, a.Du, a.Dl * a.cB, a.Du * kTA, ldE, a.Du, 0, xu, a.cB, xl, kTA}, T, E, X);
   __syncthreads();
   const Product s2{a.Dl * a.Du, a.cB, a.Dr * a.Dd, ldX, ldA, a.cB, 0, yb, a.Dd, kTA, yd};
@@ -185,7 +229,12 @@ __global__ void __launch_bounds__(256) env3_f32_kernel(const Env3Fused a, float*
       load_site(slot ^ 1);
       __syncthreads();
     }
-    run<false>(s2, X, A, Y);
+    Copy cp;
+    if constexpr (MID) {
+      cp.p = mid.p + c * mid.bs + a0 * mid.sj;
+      cp.si = mid.sb; cp.sc1 = mid.sr; cp.sc2 = mid.sd; cp.sj = mid.sj; cp.nc2 = a.Dd;
+    }
+    run<false, MID>(s2, X, A, Y, 1, nj, cp);
     __syncthreads();
     run<true>(s3, Y, B, O + c * a.bsO + a0 * a.sOa2, (int)a.sOa2, nj);
     if (v == 0 && out1) __syncthreads();
@@ -280,16 +329,18 @@ bool env3_f32_fits(const Env3Fused& a) {
   return (long long)off[6] * 4 <= kMaxSmem;
 }
 
-cudaError_t env3_f32(const Env3Fused& a, float* out1, bool rev, cudaStream_t st) {
+cudaError_t env3_f32(const Env3Fused& a, float* out1, bool rev2, bool rev3, const Mid3& mid, cudaStream_t st) {
   if (g_dry_run || a.batch <= 0) return cudaSuccess;
   int off[7];
   layout3(a, off);
-  static const cudaError_t allowed = allow_smem(env3_f32_kernel);
+  static const cudaError_t allowed = allow_smem(env3_f32_kernel<false>), allowed_mid = allow_smem(env3_f32_kernel<true>);
   PV_CUDA(allowed);
+  PV_CUDA(allowed_mid);
   const long long blocks = (long long)a.batch * ((a.cT2 + kTA - 1) / kTA);
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int tasks = a.Du * ((a.Dl * a.cB + 3) / 4), tasks2 = a.cB * ((a.Dr * a.Dd + 3) / 4);
-  env3_f32_kernel<<<(unsigned)blocks, threads_for(tasks > tasks2 ? tasks : tasks2), off[6] * 4, st>>>(a, out1, rev);
+  auto* kernel = mid.p ? env3_f32_kernel<true> : env3_f32_kernel<false>;
+  kernel<<<(unsigned)blocks, threads_for(tasks > tasks2 ? tasks : tasks2), off[6] * 4, st>>>(a, out1, rev2, rev3, mid);
   return cudaGetLastError();
 }
 

@@ -57,7 +57,7 @@ extern "C" int pepsvmc_env3_left_noalloc(const float* E, const float* T, const f
   const long long no = n_chains * f.bsO;
   if (env3_f32_fits(f) && !overlaps(out, no, E, n_chains * f.bsE) && !overlaps(out, no, T, n_chains * f.bsT) &&
       !overlaps(out, no, A, 2 * f.ssA))
-    return env3_f32(f, nullptr, false, (cudaStream_t)stream) == cudaSuccess ? PEPSVMC_OK : PEPSVMC_ECUDA;
+    return env3_f32(f, nullptr, false, false, Mid3(), (cudaStream_t)stream) == cudaSuccess ? PEPSVMC_OK : PEPSVMC_ECUDA;
   float* scratch = nullptr;
   const int rc = scratch_on_current_device(&scratch);
   if (rc != PEPSVMC_OK) return rc;
