@@ -8,6 +8,11 @@
 // chain from the spin array (slot = sigma < 0), and scatters C into the layout
 // the next stage wants (up to three nested indices on each of m and n), so no
 // separate transpose kernels are needed.
+//
+// The products are small (K of a few tens, one or two tiles per chain), so a CTA's time is
+// its load latency, not its arithmetic: the next BK values of k are fetched into registers
+// while the present ones are multiplied.  Measured (1024 chains, with ~6 us of event time):
+// M 64, N 16, K 64 29.9 -> 20.7 us; M 144, N 24, K 144 with 40 chains 20.9 -> 11.7 us.
 #include "common.cuh"
 
 namespace pv {
@@ -47,22 +52,35 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(const GemmDesc d) {
 #pragma unroll
     for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
 
+  // this thread's elements of a tile of A: LA of them, dm rows and dk values of k apart
   const bool a_m_fast = (d.sAm == 1);
   const bool b_n_fast = (d.sBn == 1);
+  static_assert(256 % BM == 0 && 256 % BN == 0 && 256 % BK == 0);
+  constexpr int LA = BM * BK / 256, LB = BN * BK / 256;
+  const int am = a_m_fast ? t % BM : t / BK, ak = a_m_fast ? t / BM : t % BK;
+  const int adm = a_m_fast ? 0 : 256 / BK, adk = a_m_fast ? 256 / BM : 0;
+  const int bn = b_n_fast ? t % BN : t / BK, bk = b_n_fast ? t / BN : t % BK;
+  const int bdn = b_n_fast ? 0 : 256 / BK, bdk = b_n_fast ? 256 / BN : 0;
+  const float* pa = A + (long long)(m0 + am) * d.sAm + (long long)ak * d.sAk;
+  const float* pb = B + (long long)bk * d.sBk + (long long)(n0 + bn) * d.sBn;
+  const long long ia = adm * d.sAm + adk * d.sAk, ib = bdk * d.sBk + bdn * d.sBn;
+  float ra[LA], rb[LB];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < LA; ++q)
+      ra[q] = (m0 + am + q * adm < d.M && k0 + ak + q * adk < d.K) ? pa[k0 * d.sAk + q * ia] : 0.f;
+#pragma unroll
+    for (int q = 0; q < LB; ++q)
+      rb[q] = (n0 + bn + q * bdn < d.N && k0 + bk + q * bdk < d.K) ? pb[k0 * d.sBk + q * ib] : 0.f;
+  };
+  fetch(0);
   for (int k0 = 0; k0 < d.K; k0 += BK) {
-    for (int i = t; i < BM * BK; i += 256) {
-      int mm, kk;
-      if (a_m_fast) { mm = i % BM; kk = i / BM; } else { kk = i % BK; mm = i / BK; }
-      const int m = m0 + mm, k = k0 + kk;
-      As[kk][mm] = (m < d.M && k < d.K) ? A[(long long)m * d.sAm + (long long)k * d.sAk] : 0.f;
-    }
-    for (int i = t; i < BN * BK; i += 256) {
-      int nn, kk;
-      if (b_n_fast) { nn = i % BN; kk = i / BN; } else { kk = i % BK; nn = i / BK; }
-      const int n = n0 + nn, k = k0 + kk;
-      Bs[kk][nn] = (n < d.N && k < d.K) ? B[(long long)k * d.sBk + (long long)n * d.sBn] : 0.f;
-    }
+#pragma unroll
+    for (int q = 0; q < LA; ++q) As[ak + q * adk][am + q * adm] = ra[q];
+#pragma unroll
+    for (int q = 0; q < LB; ++q) Bs[bk + q * bdk][bn + q * bdn] = rb[q];
     __syncthreads();
+    if (k0 + BK < d.K) fetch(k0 + BK);
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
       float a[TM], bb[TN];
