@@ -15,15 +15,19 @@
 // The optimal site of the boundary-MPS fit is the same chain of products with a boundary bond
 // in the place of a'; its middle product goes to memory as well, where the product that
 // makes the next environment reads it (fit of Dc 16, D 4, 1024 chains: 92 us in three products,
-// 41 us in one kernel, with ~6 us of event time per launch).
+// 32 us in one kernel, with ~6 us of event time per launch).
 //
 // Bound: FP32 arithmetic.  The separate products wrote and read every intermediate through
 // global memory, 4 bytes per 32-byte sector where the next product wanted another order, and
-// waited for their loads at every 16 values of k.  Measured (separate -> fused): three-line
-// step Dc 24, D 6, 2048 chains 909 -> 350 us (20 TFLOP/s), Dc 16, D 4, 1024 chains 80 -> 27 us,
-// Dc 32, D 8, 512 chains 578 -> 322 us, 64 chains of Dc 16, D 4 28 -> 11 us; four-line step
-// Dc 16, D 4, 1024 chains 385 -> 101 us.  Steps whose intermediates exceed a CTA's shared
-// memory keep the separate products.
+// waited for their loads.  Here all operands of a step are in flight at once, by asynchronous
+// copies (through registers, in turn, a third of the time went to loading: Dc 24, D 6 350 us,
+// and odd bonds, one CTA per SM, were slower than the separate products: Dc 25, D 7, 40 chains
+// 65 us against 40).  Measured (separate -> fused): three-line step Dc 24, D 6, 2048 chains
+// 909 -> 244 us (29 TFLOP/s), Dc 16, D 4, 1024 chains 80 -> 21 us, Dc 32, D 8, 512 chains 578 ->
+// 262 us, Dc 23, D 7, 1624 chains 741 -> 486 us, 64 chains of Dc 16, D 4 28 -> 9 us; four-line step
+// Dc 16, D 4, 1024 chains 385 -> 86 us, Dc 17, D 5, 104 chains 99 -> 85 us.  Over 120 drawn steps
+// (bonds to 32 and 8, 1-2048 chains) 118 are at 1.0x or above, the others at 0.91 and 0.99.
+// Steps whose intermediates exceed a CTA's shared memory keep the separate products.
 #include "fused_f32.cuh"
 
 namespace pv {
@@ -137,42 +141,72 @@ __device__ __forceinline__ void run(const Product& g, const float* p, const floa
   else product<4, 2, GLOBAL, COPY>(g, p, q, o, sj, nj, cp);
 }
 
+// Operands come in by asynchronous copies, all of a step's in flight at once; loads_done waits
+// for this thread's (before the barrier that precedes their use).
+template <int BYTES>
+__device__ __forceinline__ void copy_async(float* dst, const float* src, bool valid = true) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  if constexpr (BYTES == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(valid ? 16 : 0) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void loads_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// The threads as rows of 1 to 32 lanes (a power of two that covers n, if 32 do).
+struct Rows {
+  int lanes, lane, row, rows;
+  __device__ __forceinline__ explicit Rows(int n) {
+    const int lg = n >= 32 ? 5 : 32 - __clz(n - 1);
+    lanes = 1 << lg;
+    lane = threadIdx.x & (lanes - 1);
+    row = threadIdx.x >> lg;
+    rows = blockDim.x >> lg;
+  }
+};
+
 // dst[k*ld + c] for k < n0 * n1 (n0 outer), c < nc, c = (c / nc2, c % nc2), zero up to ld.
 __device__ __forceinline__ void load_cols(float* dst, int ld, const float* src, int n0, int s0, int n1, int s1, int nc,
                                           int nc2, int sc1, int sc2) {
+  const bool row = sc2 == 1 && (nc == nc2 || sc1 == nc2);  // rows contiguous
   // a dense block in the same order: 16-byte copies
-  if (ld == nc && sc2 == 1 && (nc == nc2 || sc1 == nc2) && (n1 == 1 || s1 == nc) && s0 == n1 * nc && (nc & 3) == 0 &&
-      (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+  if (ld == nc && row && (n1 == 1 || s1 == nc) && s0 == n1 * nc && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
     const int n = n0 * n1 * nc / 4;
-    for (int e = threadIdx.x; e < n; e += blockDim.x)
-      reinterpret_cast<float4*>(dst)[e] = reinterpret_cast<const float4*>(src)[e];
-    return;
-  }
-  const int n = n0 * n1 * ld;
-  if (n1 == 1 && s0 == 1 && sc2 != 1) {  // k contiguous (a mirrored view): lanes along k
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-      const int k = e % n0, c = e / n0;
-      dst[k * ld + c] = c < nc ? src[k + (c / nc2) * sc1 + (c % nc2) * sc2] : 0.f;
+    for (int e = threadIdx.x; e < n; e += blockDim.x) copy_async<16>(dst + 4 * e, src + 4 * e);
+  } else if (n1 == 1 && s0 == 1 && sc2 != 1) {  // k contiguous (a mirrored view): lanes along k
+    const Rows t(n0);
+    for (int c = t.row; c < ld; c += t.rows) {
+      const float* p = src + (c < nc ? (c / nc2) * sc1 + (c % nc2) * sc2 : 0);
+      for (int k = t.lane; k < n0; k += t.lanes) copy_async<4>(dst + k * ld + c, p + k, c < nc);
     }
-    return;
-  }
-  for (int e = threadIdx.x; e < n; e += blockDim.x) {
-    const int c = e % ld, k = e / ld;
-    dst[e] = c < nc ? src[(k / n1) * s0 + (k % n1) * s1 + (c / nc2) * sc1 + (c % nc2) * sc2] : 0.f;
+  } else {
+    const Rows t(ld);
+    for (int k = t.row; k < n0 * n1; k += t.rows) {
+      const float* p = src + (n1 == 1 ? k * s0 : (k / n1) * s0 + (k % n1) * s1);
+      for (int c = t.lane; c < ld; c += t.lanes)
+        copy_async<4>(dst + k * ld + c, c < nc ? p + (row ? c : (c / nc2) * sc1 + (c % nc2) * sc2) : src, c < nc);
+    }
   }
 }
 // T tile: dst[(a*Du + u)*8 + j], zero beyond the bond.
 __device__ __forceinline__ void load_top(float* dst, const float* T, int cT, int Du, int sTa, int sTu, int sTa2, int nj) {
   const int n = cT * Du * kTA;
-  if (sTa2 == 1 || sTa != 1) {
+  if (sTa2 == 1 && nj == kTA && ((reinterpret_cast<uintptr_t>(T) | (sTa | sTu) * 4) & 15) == 0) {
+    for (int e = threadIdx.x; e < n / 4; e += blockDim.x) {
+      const int au = e >> 1, a = au / Du;
+      copy_async<16>(dst + 4 * e, T + a * sTa + (au - a * Du) * sTu + (e & 1) * 4);
+    }
+  } else if (sTa2 == 1 || sTa != 1) {
     for (int e = threadIdx.x; e < n; e += blockDim.x) {
-      const int j = e % kTA, au = e / kTA;
-      dst[e] = j < nj ? T[(au / Du) * sTa + (au % Du) * sTu + j * sTa2] : 0.f;
+      const int j = e % kTA, au = e / kTA, a = au / Du;
+      copy_async<4>(dst + e, j < nj ? T + a * sTa + (au - a * Du) * sTu + j * sTa2 : T, j < nj);
     }
   } else {  // a contiguous (mirrored view): lanes along a
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-      const int a = e % cT, ju = e / cT, j = ju / Du, u = ju % Du;
-      dst[(a * Du + u) * kTA + j] = j < nj ? T[a + u * sTu + j * sTa2] : 0.f;
+    const Rows t(cT);
+    for (int ju = t.row; ju < kTA * Du; ju += t.rows) {
+      const int j = ju / Du, u = ju - j * Du;
+      for (int a = t.lane; a < cT; a += t.lanes)
+        copy_async<4>(dst + (a * Du + u) * kTA + j, j < nj ? T + a + u * sTu + j * sTa2 : T, j < nj);
     }
   }
 }
@@ -182,23 +216,24 @@ __device__ __forceinline__ int slot_of(const int8_t* sel, long long stride, int 
   return sel ? ((sel[c * stride] < 0) ? 1 : 0) ^ flip : 0;
 }
 
-// Floats of shared memory: E, T, A, B, X, Y.
-__host__ __device__ inline void layout3(const Env3Fused& a, int off[7]) {
+// Floats of shared memory: E, T, A, B, X; Y takes the place of E and T, which only the first
+// product reads.
+__host__ __device__ inline int layout3(const Env3Fused& a, int off[5]) {
+  const int t = a.cT * pad4(a.Dl * a.cB), et = t + a.cT * a.Du * kTA, y = a.cB * a.Dd * a.Dr * kTA;
   off[0] = 0;
-  off[1] = off[0] + a.cT * pad4(a.Dl * a.cB);
-  off[2] = off[1] + a.cT * a.Du * kTA;
+  off[1] = t;
+  off[2] = et > y ? et : y;
   off[3] = off[2] + a.Dl * a.Du * pad4(a.Dr * a.Dd);
   off[4] = off[3] + a.cB * a.Dd * pad4(a.cB2);
-  off[5] = off[4] + a.Dl * a.Du * a.cB * kTA;
-  off[6] = off[5] + a.cB * a.Dd * a.Dr * kTA;
+  return off[4] + a.Dl * a.Du * a.cB * kTA;
 }
 
 template <bool MID>
-__global__ void __launch_bounds__(256, MID ? 3 : 0) env3_f32_kernel(const Env3Fused a, float* out1, bool rev2, bool rev3, const Mid3 mid) {
+__global__ void __maxnreg__(80) env3_f32_kernel(const Env3Fused a, float* out1, bool rev2, bool rev3, const Mid3 mid) {
   extern __shared__ __align__(16) float sf[];
-  int off[7];
+  int off[5];
   layout3(a, off);
-  float *E = sf + off[0], *T = sf + off[1], *A = sf + off[2], *B = sf + off[3], *X = sf + off[4], *Y = sf + off[5];
+  float *E = sf + off[0], *T = sf + off[1], *A = sf + off[2], *B = sf + off[3], *X = sf + off[4], *Y = sf;
   const int n_at = (a.cT2 + kTA - 1) / kTA, c = blockIdx.x / n_at, a0 = (blockIdx.x % n_at) * kTA;
   const int nj = min(kTA, a.cT2 - a0);
   const int slot = slot_of(a.sel, a.sel_stride, a.sel_xor, c);
@@ -214,6 +249,7 @@ __global__ void __launch_bounds__(256, MID ? 3 : 0) env3_f32_kernel(const Env3Fu
   load_site(slot);
   if (rev3) load_cols(B, ldB, a.B + c * a.bsB, a.Dd, (int)a.sBd, a.cB, (int)a.sBb, a.cB2, a.cB2, 0, (int)a.sBb2);
   else load_cols(B, ldB, a.B + c * a.bsB, a.cB, (int)a.sBb, a.Dd, (int)a.sBd, a.cB2, a.cB2, 0, (int)a.sBb2);
+  loads_done();
   __syncthreads();
   const int ldX = a.cB * kTA, ldY = a.Dr * kTA;
   const int xl = rev2 ? ldX : a.Du * ldX, xu = rev2 ? a.Dl * ldX : ldX;
@@ -227,6 +263,7 @@ __global__ void __launch_bounds__(256, MID ? 3 : 0) env3_f32_kernel(const Env3Fu
     if (!O) break;
     if (v) {  // the other slot of the site, X shared
       load_site(slot ^ 1);
+      loads_done();
       __syncthreads();
     }
     Copy cp;
@@ -241,26 +278,27 @@ __global__ void __launch_bounds__(256, MID ? 3 : 0) env3_f32_kernel(const Env3Fu
   }
 }
 
-// Floats of shared memory: E, T, A1, A2, B, X, Y, Z; with one variant Z takes X's place.
-__host__ __device__ inline void layout4(const Env4Fused& a, bool several, int off[9]) {
+// Floats of shared memory: E, T, A1, A2, B, X, Z; Y in the place of E and T, and with one
+// variant Z in X's.
+__host__ __device__ inline int layout4(const Env4Fused& a, bool several, int off[7]) {
   const int x = a.D1l * a.Du1 * a.D2l * a.cB * kTA, z = a.cB * a.Dd2 * a.D1r * a.D2r * kTA;
+  const int t = a.cT * pad4(a.D1l * a.D2l * a.cB), et = t + a.cT * a.Du1 * kTA, y = a.D2l * a.Dd1 * a.cB * a.D1r * kTA;
   off[0] = 0;
-  off[1] = off[0] + a.cT * pad4(a.D1l * a.D2l * a.cB);
-  off[2] = off[1] + a.cT * a.Du1 * kTA;
+  off[1] = t;
+  off[2] = et > y ? et : y;
   off[3] = off[2] + a.D1l * a.Du1 * pad4(a.D1r * a.Dd1);
   off[4] = off[3] + a.D2l * a.Dd1 * pad4(a.D2r * a.Dd2);
   off[5] = off[4] + a.cB * a.Dd2 * pad4(a.cB2);
   off[6] = off[5] + (several || x > z ? x : z);
-  off[7] = off[6] + a.D2l * a.Dd1 * a.cB * a.D1r * kTA;
-  off[8] = off[7] + (several ? z : 0);
+  return off[6] + (several ? z : 0);
 }
 
-__global__ void __launch_bounds__(256) env4_f32_kernel(const Env4Fused a, const Env4Outs outs, bool several, bool rev) {
+__global__ void __maxnreg__(80) env4_f32_kernel(const Env4Fused a, const Env4Outs outs, bool several, bool rev) {
   extern __shared__ __align__(16) float sf[];
-  int off[9];
+  int off[7];
   layout4(a, several, off);
-  float *E = sf + off[0], *T = sf + off[1], *A1 = sf + off[2], *A2 = sf + off[3], *B = sf + off[4], *X = sf + off[5],
-        *Y = sf + off[6], *Z = several ? sf + off[7] : X;
+  float *E = sf + off[0], *T = sf + off[1], *A1 = sf + off[2], *A2 = sf + off[3], *B = sf + off[4], *X = sf + off[5], *Y = sf,
+        *Z = several ? sf + off[6] : X;
   const int n_at = (a.cT2 + kTA - 1) / kTA, c = blockIdx.x / n_at, a0 = (blockIdx.x % n_at) * kTA;
   const int nj = min(kTA, a.cT2 - a0);
   const int nE = a.D1l * a.D2l * a.cB, ldE = pad4(nE), ld1 = pad4(a.D1r * a.Dd1), ld2 = pad4(a.D2r * a.Dd2),
@@ -289,6 +327,7 @@ __global__ void __launch_bounds__(256) env4_f32_kernel(const Env4Fused a, const 
   for (int f1 = 0; f1 < 2; ++f1) {
     if (!outs.p[2 * f1] && !outs.p[2 * f1 + 1]) continue;
     load1(slot1 ^ f1);
+    loads_done();
     __syncthreads();
     // X(l1,u1 | l2,b): columns (l1, (l2,b)), rows u1
     if (fresh) {
@@ -302,6 +341,7 @@ __global__ void __launch_bounds__(256) env4_f32_kernel(const Env4Fused a, const 
       float* O = outs.p[2 * f1 + f2];
       if (!O) continue;
       load2(slot2 ^ f2);
+      loads_done();
       __syncthreads();
       // Z(b,d2 | r1,r2): rows (b, r1), columns (r2, d2)
       run<false>(Product{a.D2l * a.Dd1, a.cB * a.D1r, a.D2r * a.Dd2, ldY, ld2, a.D1r, zb, a.D2r * kTA, a.Dd2, kTA, zd}, Y, A2, Z);
@@ -313,8 +353,11 @@ __global__ void __launch_bounds__(256) env4_f32_kernel(const Env4Fused a, const 
   }
 }
 
-// Threads of a CTA: enough for the first products' tasks of 8 x 4, at most 256.
-int threads_for(int tasks) { return tasks > 128 ? 256 : tasks > 64 ? 128 : 64; }
+// Threads of a CTA: enough for the first products' tasks of 8 x 4, at most 256, or 512 where the
+// shared memory lets an SM hold one CTA only.
+int threads_for(int tasks, int smem) {
+  return tasks > 256 && 2 * (smem + 1024) > 228 * 1024 ? 512 : tasks > 128 ? 256 : tasks > 64 ? 128 : 64;
+}
 
 template <typename K>
 cudaError_t allow_smem(K kernel) {
@@ -324,15 +367,14 @@ cudaError_t allow_smem(K kernel) {
 }  // namespace
 
 bool env3_f32_fits(const Env3Fused& a) {
-  int off[7];
-  layout3(a, off);
-  return (long long)off[6] * 4 <= kMaxSmem;
+  int off[5];
+  return (long long)layout3(a, off) * 4 <= kMaxSmem;
 }
 
 cudaError_t env3_f32(const Env3Fused& a, float* out1, bool rev2, bool rev3, const Mid3& mid, cudaStream_t st) {
   if (g_dry_run || a.batch <= 0) return cudaSuccess;
-  int off[7];
-  layout3(a, off);
+  int off[5];
+  const int smem = layout3(a, off) * 4;
   static const cudaError_t allowed = allow_smem(env3_f32_kernel<false>), allowed_mid = allow_smem(env3_f32_kernel<true>);
   PV_CUDA(allowed);
   PV_CUDA(allowed_mid);
@@ -340,28 +382,27 @@ cudaError_t env3_f32(const Env3Fused& a, float* out1, bool rev2, bool rev3, cons
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int tasks = a.Du * ((a.Dl * a.cB + 3) / 4), tasks2 = a.cB * ((a.Dr * a.Dd + 3) / 4);
   auto* kernel = mid.p ? env3_f32_kernel<true> : env3_f32_kernel<false>;
-  kernel<<<(unsigned)blocks, threads_for(tasks > tasks2 ? tasks : tasks2), off[6] * 4, st>>>(a, out1, rev2, rev3, mid);
+  kernel<<<(unsigned)blocks, threads_for(tasks > tasks2 ? tasks : tasks2, smem), smem, st>>>(a, out1, rev2, rev3, mid);
   return cudaGetLastError();
 }
 
 static bool several(const Env4Outs& o) { return (o.p[0] != nullptr) + (o.p[1] != nullptr) + (o.p[2] != nullptr) + (o.p[3] != nullptr) > 1; }
 
 bool env4_f32_fits(const Env4Fused& a, const Env4Outs& outs) {
-  int off[9];
-  layout4(a, several(outs), off);
-  return a.sEl1 == (long long)a.D2l * a.sEl2 && (long long)off[8] * 4 <= kMaxSmem;
+  int off[7];
+  return a.sEl1 == (long long)a.D2l * a.sEl2 && (long long)layout4(a, several(outs), off) * 4 <= kMaxSmem;
 }
 
 cudaError_t env4_f32(const Env4Fused& a, const Env4Outs& outs, bool rev, cudaStream_t st) {
   if (g_dry_run || a.batch <= 0) return cudaSuccess;
-  int off[9];
-  layout4(a, several(outs), off);
+  int off[7];
+  const int smem = layout4(a, several(outs), off) * 4;
   static const cudaError_t allowed = allow_smem(env4_f32_kernel);
   PV_CUDA(allowed);
   const long long blocks = (long long)a.batch * ((a.cT2 + kTA - 1) / kTA);
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int tasks = a.D2l * a.cB * ((a.D1r * a.Dd1 + 3) / 4);
-  env4_f32_kernel<<<(unsigned)blocks, threads_for(tasks), off[8] * 4, st>>>(a, outs, several(outs), rev);
+  env4_f32_kernel<<<(unsigned)blocks, threads_for(tasks, smem), smem, st>>>(a, outs, several(outs), rev);
   return cudaGetLastError();
 }
 

@@ -34,6 +34,7 @@ def context(n, D, chi):
     (33, 9, 7, 11, 13, 3, 2, 4, 2),      # every bond different, no extent a multiple of 4
     (5, 1, 1, 1, 1, 1, 1, 1, 1),
     (7, 4, 16, 9, 3, 4, 1, 4, 4),
+    (6, 25, 29, 27, 31, 7, 8, 8, 7),     # 512 threads, rows that no 16-byte copy takes
 ])
 def test_env3_equals_separate_products(torch_mod, n, cT, cB, cT2, cB2, Dl, Dr, Du, Dd):
     torch = torch_mod
@@ -70,6 +71,7 @@ def test_env3_equals_separate_products(torch_mod, n, cT, cB, cT2, cB2, Dl, Dr, D
     (11, 9, 7, 11, 13, 3, 2, 4, 2, 3, 2, 2),
     (3, 1, 1, 4, 3, 1, 4, 1, 4, 1, 4, 4),
     (4, 20, 13, 19, 9, 5, 3, 4, 5, 2, 5, 3),
+    (5, 17, 17, 17, 17, 5, 5, 5, 5, 5, 5, 5),  # 512 threads, rows that no 16-byte copy takes
 ])
 def test_env4_equals_separate_products(torch_mod, n, cT, cB, cT2, cB2, D1l, D1r, Du1, Dd1, D2l, D2r, Dd2):
     torch = torch_mod
@@ -90,7 +92,8 @@ def test_env4_equals_separate_products(torch_mod, n, cT, cB, cT2, cB2, D1l, D1r,
     ctx.close()
 
 
-@pytest.mark.parametrize("Ly,Lx,D,chi,J2", [(4, 6, 3, 10, 0.5), (6, 4, 5, 17, 0.5), (4, 4, 4, 16, 0.0)])
+@pytest.mark.parametrize("Ly,Lx,D,chi,J2", [(4, 6, 3, 10, 0.5), (6, 4, 5, 17, 0.5), (4, 4, 4, 16, 0.0),
+                                             (4, 6, 8, 26, 0.0)])
 def test_sweep_and_measurement_have_the_same_bits(torch_mod, Ly, Lx, D, chi, J2):
     from paper_1908_09359_gb300 import api
     t = inputs.peps_tensors(Ly, Lx, D, 5, True, bond_decay=1.0)
