@@ -27,16 +27,17 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(const GemmDesc d) {
   __shared__ __align__(16) float Bs[BK][BN + 4];
   __shared__ long long s_on[BN];  // C offset of each tile column (the same for every row)
 
+  after_previous();
   const int b = blockIdx.y + blockIdx.z * gridDim.y;
   if (b >= d.batch) return;
   const int tiles_n = (d.N + BN - 1) / BN;
   const int m0 = (blockIdx.x / tiles_n) * BM;
   const int n0 = (blockIdx.x % tiles_n) * BN;
 
-  const float* __restrict__ A = d.A + (long long)b * d.bsA;
+  const float* A = d.A + (long long)b * d.bsA;
   long long boff = (long long)b * d.bsB;
   if (d.sel) boff += (long long)(((d.sel[(long long)b * d.sel_stride] < 0) ? 1 : 0) ^ d.sel_xor) * d.ssB;
-  const float* __restrict__ B = d.B + boff;
+  const float* B = d.B + boff;
 
   const int t = threadIdx.x;
   const int tx = t % TX, ty = t / TX;
@@ -150,8 +151,7 @@ template <int BM, int BN, int TM, int TN>
 cudaError_t launch(const GemmDesc& d, cudaStream_t st) {
   const int tiles = ((d.M + BM - 1) / BM) * ((d.N + BN - 1) / BN);
   dim3 grid(tiles, d.batch < 65535 ? d.batch : 65535, (d.batch + 65534) / 65535);
-  gemm_f32_kernel<BM, BN, 16, TM, TN><<<grid, 256, 0, st>>>(d);
-  return cudaGetLastError();
+  return launch_early(gemm_f32_kernel<BM, BN, 16, TM, TN>, grid, 256, 0, st, d);
 }
 
 }  // namespace

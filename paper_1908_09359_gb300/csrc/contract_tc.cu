@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const GemmDesc d, uns
   __shared__ uint32_t tmem_base;
   __shared__ long long s_on[BN];  // C offset of each tile column (the same for every row)
 
+  after_previous();
   const int b = blockIdx.y + blockIdx.z * gridDim.y;
   if (b >= d.batch) return;
   const int tiles_n = (d.N + BN - 1) / BN;
@@ -298,8 +299,7 @@ cudaError_t launch(const GemmDesc& d, unsigned* status, cudaStream_t st) {
   }
   const int tiles = ((d.M + kBM - 1) / kBM) * ((d.N + BN - 1) / BN);
   dim3 grid(tiles, d.batch < 65535 ? d.batch : 65535, (d.batch + 65534) / 65535);
-  gemm_tc_kernel<EB, BN, X3, DB><<<grid, kThreads, smem, st>>>(d, status);
-  return cudaGetLastError();
+  return launch_early(gemm_tc_kernel<EB, BN, X3, DB>, grid, kThreads, smem, st, d, status);
 }
 
 template <int EB, bool X3>

@@ -386,6 +386,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) env3_fused_kernel(const __gri
   tc_before_sync();
   __syncthreads();
   tc_after_sync();
+  after_previous();
   const uint32_t tmem = tmem_base;
   const PipeWait wait{&ctl};
   switch (pipe_role(warp)) {
@@ -431,8 +432,7 @@ template <bool X3, bool FULL>
 cudaError_t launch(const Plan3& P, int grid, unsigned* status, cudaStream_t st) {
   static const cudaError_t configured = configure(env3_fused_kernel<X3, FULL>, SMEM_BYTES);
   PV_CUDA(configured);
-  env3_fused_kernel<X3, FULL><<<grid, kPipeThreads, SMEM_BYTES, st>>>(P, status);
-  return cudaGetLastError();
+  return launch_early(env3_fused_kernel<X3, FULL>, grid, kPipeThreads, SMEM_BYTES, st, P, status);
 }
 
 // ------------------------------------------------------------ optimal site of the fit
@@ -695,6 +695,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) proj3_fused_kernel(const __gr
   tc_before_sync();
   __syncthreads();
   tc_after_sync();
+  after_previous();
   const uint32_t tmem = tmem_base;
   const PipeWait wait{&ctl};
   switch (pipe_role(warp)) {
@@ -727,8 +728,7 @@ template <bool X3, bool FULL>
 cudaError_t launch_proj3(const PlanP& P, int grid, unsigned* status, cudaStream_t st) {
   static const cudaError_t configured = configure(proj3_fused_kernel<X3, FULL>, P_SMEM_BYTES);
   PV_CUDA(configured);
-  proj3_fused_kernel<X3, FULL><<<grid, kPipeThreads, P_SMEM_BYTES, st>>>(P, status);
-  return cudaGetLastError();
+  return launch_early(proj3_fused_kernel<X3, FULL>, grid, kPipeThreads, P_SMEM_BYTES, st, P, status);
 }
 
 bool all_full(const PipeOp (&op)[4]) {

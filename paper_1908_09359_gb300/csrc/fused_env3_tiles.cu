@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(kThreads, 2) env3_tile_kernel(const Env3Fused 
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(sm);
 
+  after_previous();
   const int n_at = (a.cT2 + kAT - 1) / kAT, n_bt = (a.cB + kBT - 1) / kBT;
   const int n_units = a.batch * n_at;
   if ((int)blockIdx.x >= n_units) return;
@@ -429,8 +430,7 @@ cudaError_t launch(const Env3Fused& a, unsigned* status, cudaStream_t st) {
   const long long units = (long long)a.batch * ((a.cT2 + kAT - 1) / kAT);
   if (units > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = (int)(units < ctas ? units : ctas);
-  env3_tile_kernel<X3><<<grid, kThreads, SMEM_BYTES, st>>>(a, status);
-  return cudaGetLastError();
+  return launch_early(env3_tile_kernel<X3>, grid, kThreads, SMEM_BYTES, st, a, status);
 }
 
 // ------------------------------------------------------------ optimal site of the fit
@@ -541,6 +541,7 @@ __global__ void __launch_bounds__(kThreads, 2) proj3_tile_kernel(const Proj3Fuse
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(sm);
 
+  after_previous();
   const int n_vt = (a.cV + kPV - 1) / kPV, n_at = (a.cT2 + kAT - 1) / kAT;
   const int n_units = a.batch * n_vt;
   if ((int)blockIdx.x >= n_units) return;
@@ -719,8 +720,7 @@ cudaError_t launch_proj3(const Proj3Fused& a, unsigned* status, cudaStream_t st)
   const long long units = (long long)a.batch * ((a.cV + kPV - 1) / kPV);
   if (units > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = (int)(units < ctas ? units : ctas);
-  proj3_tile_kernel<X3><<<grid, kThreads, P_SMEM_BYTES, st>>>(a, status);
-  return cudaGetLastError();
+  return launch_early(proj3_tile_kernel<X3>, grid, kThreads, P_SMEM_BYTES, st, a, status);
 }
 
 }  // namespace

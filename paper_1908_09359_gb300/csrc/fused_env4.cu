@@ -137,6 +137,7 @@ __global__ void __launch_bounds__(kThreads, 2) env4_fused_kernel(const Env4Fused
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(sm);
 
+  after_previous();
   const int n_at = (a.cT2 + kAT - 1) / kAT, n_bt = (a.cB + kBT - 1) / kBT;
   const int c = blockIdx.x / n_at, t = blockIdx.x % n_at;
   if (c >= a.batch) return;
@@ -347,8 +348,7 @@ cudaError_t launch(const Env4Fused& a, unsigned* status, cudaStream_t st) {
   }
   const long long blocks = (long long)a.batch * ((a.cT2 + kAT - 1) / kAT);
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-  env4_fused_kernel<X3><<<(unsigned)blocks, kThreads, SMEM_BYTES, st>>>(a, status);
-  return cudaGetLastError();
+  return launch_early(env4_fused_kernel<X3>, (unsigned)blocks, kThreads, SMEM_BYTES, st, a, status);
 }
 
 }  // namespace

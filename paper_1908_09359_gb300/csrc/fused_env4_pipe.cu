@@ -418,6 +418,7 @@ __global__ void __launch_bounds__(kThreads, 1) env4_pipe_kernel(const __grid_con
   tc_before_sync();
   __syncthreads();
   tc_after_sync();
+  after_previous();
   const uint32_t tmem = tmem_base;
   const PipeWait wait{&ctl};
   constexpr int LOAD0 = kStreams * kDrainWarps, COPY0 = LOAD0 + kLoadWarps;
@@ -460,8 +461,7 @@ cudaError_t launch(const Plan4& P, int grid, unsigned* status, cudaStream_t st) 
   static const cudaError_t configured =
       cudaFuncSetAttribute(env4_pipe_kernel<X3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
   PV_CUDA(configured);
-  env4_pipe_kernel<X3><<<grid, kThreads, SMEM_BYTES, st>>>(P, status);
-  return cudaGetLastError();
+  return launch_early(env4_pipe_kernel<X3>, grid, kThreads, SMEM_BYTES, st, P, status);
 }
 
 }  // namespace

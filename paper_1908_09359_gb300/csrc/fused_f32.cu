@@ -236,6 +236,7 @@ __global__ void __maxnreg__(80) env3_f32_kernel(const Env3Fused a, float* out1, 
   float *E = sf + off[0], *T = sf + off[1], *A = sf + off[2], *B = sf + off[3], *X = sf + off[4], *Y = sf;
   const int n_at = (a.cT2 + kTA - 1) / kTA, c = blockIdx.x / n_at, a0 = (blockIdx.x % n_at) * kTA;
   const int nj = min(kTA, a.cT2 - a0);
+  after_previous();
   const int slot = slot_of(a.sel, a.sel_stride, a.sel_xor, c);
   const int ldE = pad4(a.Dl * a.cB), ldA = pad4(a.Dr * a.Dd), ldB = pad4(a.cB2);
   const int sAl = (int)a.sAl, sAu = (int)a.sAu, sAr = (int)a.sAr, sAd = (int)a.sAd;
@@ -303,6 +304,7 @@ __global__ void __maxnreg__(80) env4_f32_kernel(const Env4Fused a, const Env4Out
   const int nj = min(kTA, a.cT2 - a0);
   const int nE = a.D1l * a.D2l * a.cB, ldE = pad4(nE), ld1 = pad4(a.D1r * a.Dd1), ld2 = pad4(a.D2r * a.Dd2),
             ldB = pad4(a.cB2);
+  after_previous();
   const int slot1 = slot_of(a.sel1, a.sel_stride, a.xor1, c), slot2 = slot_of(a.sel2, a.sel_stride, a.xor2, c);
   auto load1 = [&](int s) {
     const float* src = a.A1 + s * a.ss1;
@@ -382,8 +384,7 @@ cudaError_t env3_f32(const Env3Fused& a, float* out1, bool rev2, bool rev3, cons
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int tasks = a.Du * ((a.Dl * a.cB + 3) / 4), tasks2 = a.cB * ((a.Dr * a.Dd + 3) / 4);
   auto* kernel = mid.p ? env3_f32_kernel<true> : env3_f32_kernel<false>;
-  kernel<<<(unsigned)blocks, threads_for(tasks > tasks2 ? tasks : tasks2, smem), smem, st>>>(a, out1, rev2, rev3, mid);
-  return cudaGetLastError();
+  return launch_early(kernel, (unsigned)blocks, threads_for(tasks > tasks2 ? tasks : tasks2, smem), smem, st, a, out1, rev2, rev3, mid);
 }
 
 static bool several(const Env4Outs& o) { return (o.p[0] != nullptr) + (o.p[1] != nullptr) + (o.p[2] != nullptr) + (o.p[3] != nullptr) > 1; }
@@ -402,8 +403,7 @@ cudaError_t env4_f32(const Env4Fused& a, const Env4Outs& outs, bool rev, cudaStr
   const long long blocks = (long long)a.batch * ((a.cT2 + kTA - 1) / kTA);
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int tasks = a.D2l * a.cB * ((a.D1r * a.Dd1 + 3) / 4);
-  env4_f32_kernel<<<(unsigned)blocks, threads_for(tasks, smem), smem, st>>>(a, outs, several(outs), rev);
-  return cudaGetLastError();
+  return launch_early(env4_f32_kernel, (unsigned)blocks, threads_for(tasks, smem), smem, st, a, outs, several(outs), rev);
 }
 
 }  // namespace pv

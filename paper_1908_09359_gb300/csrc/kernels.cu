@@ -183,6 +183,7 @@ __global__ void normalize_pow2_kernel(float* x, long long bs, int n, float* x2, 
   namespace cg = cooperative_groups;
   __shared__ float red[kThreads / 32];
   __shared__ float part;  // this block's max, NaN when an entry is not finite
+  after_previous();
   int b = blockIdx.x, blocks = 1, rank = 0, off = 0, len = n;
   if constexpr (CLUSTER) {
     blocks = cg::this_cluster().num_blocks();
@@ -251,6 +252,7 @@ __global__ void normalize_pow2_kernel(float* x, long long bs, int n, float* x2, 
 __global__ void mps_normalize_kernel(float* x, long long bs, int n, const int* exps, const double* log_in,
                                      double* log_out, unsigned* status) {
   __shared__ double red[kThreads / 32];
+  after_previous();
   const int b = blockIdx.x;
   float* xb = x + b * bs;
   double s = part_dot(xb, xb, n);
@@ -286,6 +288,7 @@ __global__ void metropolis_kernel(const MetropolisArgs a) {
   __shared__ double red[kThreads / 32];
   __shared__ float redf[kThreads / 32];
   __shared__ int acc_s;
+  after_previous();
   const int b = blockIdx.x;
   const float* cur = a.cur + b * a.bs_cur;
   const float* Rc = a.Rcur + b * a.bs_Rcur;
@@ -449,6 +452,7 @@ __device__ __forceinline__ int chain_of(int* blocks, int* rank) {
 template <bool CLUSTER>
 __global__ void dot_kernel(const float* a, long long bsa, const float* bb, long long bsb, int n, double* out,
                            unsigned* status) {
+  after_previous();
   int blocks, rank;
   const int b = chain_of<CLUSTER>(&blocks, &rank);
   const double s = chain_dot<CLUSTER>(a + b * bsa, bb + b * bsb, n, blocks, rank);
@@ -464,6 +468,7 @@ __global__ void ratio_accum_kernel(const float* a, long long bsa, const float* b
                                    const double* den, const int8_t* spins, long long spin_stride, int si, int sj,
                                    double halfJ, double* eloc, unsigned* status, float* rho_out, long long rho_stride,
                                    long long rho_idx) {
+  after_previous();
   int blocks, rank;
   const int b = chain_of<CLUSTER>(&blocks, &rank);
   const int8_t* sp = spins + b * spin_stride;
@@ -482,19 +487,20 @@ template <typename... Par, typename... Arg>
 cudaError_t launch_chains(void (*one)(Par...), void (*cluster)(Par...), int n, int batch, cudaStream_t st, Arg... arg) {
   const int c = cluster_for(n);
   if (c == 1 || batch > 0x7fffffff / c) {
-    one<<<batch, kThreads, 0, st>>>(arg...);
-    return cudaGetLastError();
+    return launch_early(one, batch, kThreads, 0, st, arg...);
   }
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = c;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = c;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(batch * c);
   cfg.blockDim = dim3(kThreads);
   cfg.stream = st;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = plain_launches(st) ? 1 : 2;
   return cudaLaunchKernelEx(&cfg, cluster, arg...);
 }
 
@@ -719,13 +725,11 @@ cudaError_t k_normalize_pow2(float* x, long long bs, int n, float* x2, long long
 cudaError_t k_mps_normalize(float* x, long long bs, int n, const int* exps, const double* log_in, double* log_out,
                             int batch, unsigned* status, cudaStream_t st) {
   if (g_dry_run) return cudaSuccess;
-  mps_normalize_kernel<<<batch, kThreads, 0, st>>>(x, bs, n, exps, log_in, log_out, status);
-  return cudaGetLastError();
+  return launch_early(mps_normalize_kernel, batch, kThreads, 0, st, x, bs, n, exps, log_in, log_out, status);
 }
 cudaError_t k_metropolis(const MetropolisArgs& a, int batch, cudaStream_t st) {
   if (g_dry_run) return cudaSuccess;
-  metropolis_kernel<<<batch, kThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_early(metropolis_kernel, batch, kThreads, 0, st, a);
 }
 cudaError_t k_phi_decide(const MetropolisArgs& a, int batch, cudaStream_t st) {
   if (g_dry_run) return cudaSuccess;

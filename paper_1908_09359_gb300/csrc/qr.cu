@@ -349,6 +349,7 @@ __global__ void __launch_bounds__(32 * W, (RPT == 4 ? 8 : 16) / W) qr_pos_tree_k
                                                              long long qcs, int R, int C) {
   using T = QrTree<RPT, W, NB>;
   __shared__ __align__(16) typename T::Smem sm;
+  after_previous();
   const int tid = threadIdx.x;
   const float* Yb = Y + (long long)blockIdx.x * bsY;
   float a[RPT][T::NC];
@@ -410,12 +411,11 @@ template <int RPT, int W>
 cudaError_t launch_tree(const float* Y, long long bsY, long long yrs, long long ycs, float* Q, long long bsQ,
                         long long qrs, long long qcs, int rows, int cols, int batch, cudaStream_t st) {
   switch ((cols + 7) / 8) {
-    case 1: qr_pos_tree_kernel<RPT, W, 1><<<batch, 32 * W, 0, st>>>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols); break;
-    case 2: qr_pos_tree_kernel<RPT, W, 2><<<batch, 32 * W, 0, st>>>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols); break;
-    case 3: qr_pos_tree_kernel<RPT, W, 3><<<batch, 32 * W, 0, st>>>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols); break;
-    default: qr_pos_tree_kernel<RPT, W, 4><<<batch, 32 * W, 0, st>>>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols); break;
+    case 1: return launch_early(qr_pos_tree_kernel<RPT, W, 1>, batch, 32 * W, 0, st, Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols);
+    case 2: return launch_early(qr_pos_tree_kernel<RPT, W, 2>, batch, 32 * W, 0, st, Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols);
+    case 3: return launch_early(qr_pos_tree_kernel<RPT, W, 3>, batch, 32 * W, 0, st, Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols);
+    default: return launch_early(qr_pos_tree_kernel<RPT, W, 4>, batch, 32 * W, 0, st, Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace
@@ -430,10 +430,8 @@ cudaError_t qr_pos_batched(const float* Y, long long bsY, long long yrs, long lo
     // matrices of the full width (304 matrices on 152 SMs; figures above)
     if (rows <= 64) return launch_tree<2, 1>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols, batch, st);
     if (rows <= 128) return launch_tree<2, 2>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols, batch, st);
-    if (cols > 24 && batch > 304) {
-      qr_pos_tree_kernel<4, 2, 4><<<batch, 64, 0, st>>>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols);
-      return cudaGetLastError();
-    }
+    if (cols > 24 && batch > 304)
+      return launch_early(qr_pos_tree_kernel<4, 2, 4>, batch, 64, 0, st, Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols);
     return launch_tree<2, 4>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols, batch, st);
   }
   const size_t smem = (size_t)2 * rows * cols * sizeof(float);
