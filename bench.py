@@ -48,11 +48,11 @@ FP32_ALU_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 # `source_sha`, per chain of that capture; the bench reports it only while the source is
 # unchanged.
 NCU_TRAFFIC = {
-    "fused4": {"bytes_per_chain": (167.906304e6 + 91.586304e6) / 512,
-               "source": "paper_1908_09359_gb300/csrc/fused_env4.cu", "source_sha": "2cb0277a6c9307e6",
+    "fused4": {"bytes_per_chain": (206.169600e6 + 98.996224e6) / 512,
+               "source": "paper_1908_09359_gb300/csrc/fused_env4_pipe.cu", "source_sha": "da40db441c68df59",
                "summary": "profiles/fused4_env4_bulk_peps24x24.md"},
-    "fused3": {"bytes_per_chain": (201.532416e6 + 45.497088e6) / 2048,
-               "source": "paper_1908_09359_gb300/csrc/fused_env3.cu", "source_sha": "49d7a78cd75df968",
+    "fused3": {"bytes_per_chain": (210.092800e6 + 45.303040e6) / 2048,
+               "source": "paper_1908_09359_gb300/csrc/fused_env3.cu", "source_sha": "103248e3ee736022",
                "summary": "profiles/fused3_env3_bulk_peps24x24.md"},
 }
 
@@ -221,13 +221,14 @@ def binding_roofline(flops, nbytes, seconds, compute_peak, hbm_peak):
 
 def kernel_groups(shapes):
     """Per-launch-shape profile records -> totals per kernel: the fused four-line and
-    three-line steps, the fit's fused optimal site, the separate tensor-core and FP32
-    products, the QR and the per-chain reductions (normalisations, ratios, decisions)."""
+    three-line steps, the fit's fused optimal site, the FP32 steps with their intermediates
+    in shared memory, the separate tensor-core and FP32 products, the QR and the per-chain reductions (normalisations, ratios, decisions)."""
     groups = {}
     for r in shapes:
         s = r["shape"]
         g = ("fused4" if s.startswith("fused4") else "fused3" if s.startswith("fused3") else
              "fusedP" if s.startswith("fusedP") else
+             "f32_fused" if s.startswith(("step3 f32", "step4 f32", "proj f32")) else
              "gemm_tc" if s.startswith("gemm tc") else "gemm_f32" if s.startswith("gemm f32") else
              "qr" if s.startswith("qr") else "reductions" if r["flops"] == 0 else "other")
         acc = groups.setdefault(g, {"launches": 0, "flops": 0.0, "ms": 0.0})
@@ -585,9 +586,10 @@ def run_ours(args):
             traffic = t["bytes_per_chain"] * C
         step_flops = prof["gemm_flops"]
         roofline = {
-            "kernel": {"fused4": "env4_fused_kernel (four-line column step, tcgen05, split BF16)",
+            "kernel": {"fused4": "env4_pipe_kernel (four-line column step, tcgen05, split BF16)",
                        "fused3": "env3_fused_kernel (three-line column step, tcgen05, split BF16)",
                        "fusedP": "proj3_fused_kernel (optimal site of the truncation fit, tcgen05, split BF16)",
+                       "f32_fused": "env3_f32_kernel, env4_f32_kernel (column steps and optimal sites, FP32 CUDA cores)",
                        "gemm_tc": "gemm_tc_kernel (separate products, tcgen05)",
                        "gemm_f32": "gemm_f32_kernel (separate products, FP32 CUDA cores)"}[dominant],
             "shape": rec["shape"], "bound": primary["bound"], "achieved": primary["achieved"],

@@ -36,7 +36,8 @@
 // tile per CTA, two CTAs per SM).
 //
 // Dc 32, D 8, split BF16, one tile per CTA -> this form: three-line step 128 chains 29.2 ->
-// 21.1 us, 512 chains 90.9 -> 52.8 us (163 TFLOP/s), 2048 chains 364 -> 176 us; optimal site of
+// 21.1 us, 512 chains 90.9 -> 52.8 us, 2048 chains 364 -> 176 us (launched early, back to back,
+// 19.7, 50.6 and 174: 109, 170 and 197 TFLOP/s; shared-memory data pipe 74 % busy); optimal site of
 // the fit 512 chains 98.8 -> 66.9 us, 128 chains 33.2 -> 25 us.  Dc 24, D 6, 2048 chains 261 ->
 // 188 us.  Tried and slower (512 chains): operands converted straight from global loads by
 // eight warps and written out by the drains, 64.5 us; by two groups of four, 90 us; all of it

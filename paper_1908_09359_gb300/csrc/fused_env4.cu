@@ -356,8 +356,8 @@ cudaError_t launch(const Env4Fused& a, unsigned* status, cudaStream_t st) {
 cudaError_t env4_fused(const Env4Fused& a, bool split, unsigned* status, cudaStream_t st) {
   if (g_dry_run || a.batch <= 0) return cudaSuccess;
   if (!env4_fused_fits(a)) return cudaErrorInvalidValue;
-  // Full bonds, b-major and dense: the pipeline, at every number of chains (61 -> 41 us at one,
-  // 566 -> 439 us at 512).  Its conversions have no bounds; smaller bonds and other orders
+  // Full bonds, b-major and dense: the pipeline, at every number of chains (61 -> 39 us at one,
+  // 566 -> 438 us at 512).  Its conversions have no bounds; smaller bonds and other orders
   // of E's indices stay with the kernel above.
   alignas(16) unsigned char plan[kEnv4PlanBytes];
   if (env4_pipe_fits(a, plan)) return env4_pipe(plan, split, status, st);

@@ -12,14 +12,15 @@
 // memory, in the order of b.  That region (128 columns) and one of 128 columns for each
 // stream's S1-S3 fill the tensor memory; a1, a2 and B are converted once per chain.
 //
-// Bound (split format): a tile's products read their operands from shared memory for ~1,770
-// cycles (128 B/cycle), its drains write for ~770, E's staging and conversion take ~400;
-// measured 3,760 cycles per tile, 78 % of that traffic's rate, the rest hand-over latency
-// (drain ~1,100 cycles, products ~1,600, beside the two other streams).  Two streams, each
-// with an S4 region of its own and E shared by two a' tiles, were at 4,150 cycles: too few
-// tiles in flight.  Measured, one-tile-per-CTA kernel -> this: 1 chain 61 -> 41 us, 76 chains
-// 87 -> 72, 128 chains 165 -> 131, 512 chains 566 -> 439, 1001 chains 1080 -> 831; plain BF16
-// 1 chain 40 -> 30, 512 chains 350 -> 293 (there the loaders set the pace).
+// Bound (split format): shared memory.  A tile's products read their operands for ~1,770 cycles
+// (128 B/cycle), its drains write for ~770, E's staging and conversion take ~400; measured
+// 3,760 cycles per tile with the data pipe 84 % busy (ncu: 40 % products, 44 % loads and
+// stores), the rest hand-over latency (drain ~1,100 cycles, products ~1,600, beside the two
+// other streams).  Two streams, each with an S4 region of its own and E shared by two a'
+// tiles, were at 4,150 cycles: too few tiles in flight.  Measured, one-tile-per-CTA kernel ->
+// this: 1 chain 61 -> 39 us, 76 chains 87 -> 72, 128 chains 165 -> 130, 512 chains 566 -> 438
+// (236 TFLOP/s), 1001 chains 1080 -> 831; plain BF16 1 chain 40 -> 30, 512 chains 350 -> 293
+// (there the loaders set the pace).
 #include <new>
 
 #include "fused.cuh"
