@@ -55,3 +55,27 @@ def test_four_line_ratios_at_full_bonds(api):
         ctx.close()
     assert np.all(np.isfinite(e[SPLIT]))
     assert np.max(np.abs(e[SPLIT] - e[0])) <= 5e-4 * max(L * L, np.max(np.abs(e[0])))
+
+
+def test_expired_waits_of_the_pipelines_return_etimeout_and_the_context_recovers(api):
+    """Full bonds and enough chains for the three- and four-line pipelines and the fit's: with a
+    budget of one clock cycle every role gives up at its first wait, what is in flight lands,
+    tensor memory is freed; with the budget restored the context gives a fresh one's bits."""
+    from paper_1908_09359_gb300._lib import PepsvmcError
+    L, n = 6, 120
+    t, sk = inputs.peps_tensors(L, L, 8, 7, True, bond_decay=1.0), inputs.sketch(L, 32, 8, 7)
+    sp = inputs.start_spins(n, L, L, 3)
+    got = []
+    for budget in (0, 1):
+        ctx = api.PepsVMC(L, L, 8, 32, n, t, sk, J2=0.5, seed=1, precision=SPLIT)
+        ctx.set_autotune(False)
+        ctx.set_spins(sp)
+        if budget:
+            ctx.set_wait_budget(budget)
+            with pytest.raises(PepsvmcError, match="ETIMEOUT"):
+                ctx.measure()
+            ctx.set_wait_budget(0)
+            ctx.set_spins(sp)
+        got.append(ctx.measure()[:2])
+        ctx.close()
+    assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
