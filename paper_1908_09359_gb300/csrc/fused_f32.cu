@@ -28,6 +28,9 @@
 // Dc 16, D 4, 1024 chains 385 -> 86 us, Dc 17, D 5, 104 chains 99 -> 85 us.  Over 120 drawn steps
 // (bonds to 32 and 8, 1-2048 chains) 118 are at 1.0x or above, the others at 0.91 and 0.99.
 // Steps whose intermediates exceed a CTA's shared memory keep the separate products.
+#include <limits.h>
+#include <math.h>
+
 #include "fused_f32.cuh"
 
 namespace pv {
@@ -211,21 +214,25 @@ __device__ __forceinline__ void load_top(float* dst, const float* T, int cT, int
   }
 }
 __host__ __device__ inline int pad4(int n) { return (n + 3) & ~3; }
+inline double pad4(double n) { return 4 * ceil(n / 4); }
 
 __device__ __forceinline__ int slot_of(const int8_t* sel, long long stride, int flip, int c) {
   return sel ? ((sel[c * stride] < 0) ? 1 : 0) ^ flip : 0;
 }
 
 // Floats of shared memory: E, T, A, B, X; Y takes the place of E and T, which only the first
-// product reads.
-__host__ __device__ inline int layout3(const Env3Fused& a, int off[5]) {
-  const int t = a.cT * pad4(a.Dl * a.cB), et = t + a.cT * a.Du * kTA, y = a.cB * a.Dd * a.Dr * kTA;
+// product reads.  N: int for a step that fits; double (whatever the bonds, no product of them wraps
+// around) where that is still to be decided.
+template <typename N>
+__host__ __device__ inline N layout3(const Env3Fused& a, N off[5]) {
+  const N cT = a.cT, cB = a.cB, cB2 = a.cB2, Dl = a.Dl, Dr = a.Dr, Du = a.Du, Dd = a.Dd;
+  const N t = cT * pad4(Dl * cB), et = t + cT * Du * kTA, y = cB * Dd * Dr * kTA;
   off[0] = 0;
   off[1] = t;
   off[2] = et > y ? et : y;
-  off[3] = off[2] + a.Dl * a.Du * pad4(a.Dr * a.Dd);
-  off[4] = off[3] + a.cB * a.Dd * pad4(a.cB2);
-  return off[4] + a.Dl * a.Du * a.cB * kTA;
+  off[3] = off[2] + Dl * Du * pad4(Dr * Dd);
+  off[4] = off[3] + cB * Dd * pad4(cB2);
+  return off[4] + Dl * Du * cB * kTA;
 }
 
 template <bool MID>
@@ -280,16 +287,19 @@ __global__ void __maxnreg__(80) env3_f32_kernel(const Env3Fused a, float* out1, 
 }
 
 // Floats of shared memory: E, T, A1, A2, B, X, Z; Y in the place of E and T, and with one
-// variant Z in X's.
-__host__ __device__ inline int layout4(const Env4Fused& a, bool several, int off[7]) {
-  const int x = a.D1l * a.Du1 * a.D2l * a.cB * kTA, z = a.cB * a.Dd2 * a.D1r * a.D2r * kTA;
-  const int t = a.cT * pad4(a.D1l * a.D2l * a.cB), et = t + a.cT * a.Du1 * kTA, y = a.D2l * a.Dd1 * a.cB * a.D1r * kTA;
+// variant Z in X's.  N as in layout3.
+template <typename N>
+__host__ __device__ inline N layout4(const Env4Fused& a, bool several, N off[7]) {
+  const N cT = a.cT, cB = a.cB, cB2 = a.cB2, D1l = a.D1l, D1r = a.D1r, Du1 = a.Du1, Dd1 = a.Dd1, D2l = a.D2l, D2r = a.D2r,
+          Dd2 = a.Dd2;
+  const N x = D1l * Du1 * D2l * cB * kTA, z = cB * Dd2 * D1r * D2r * kTA;
+  const N t = cT * pad4(D1l * D2l * cB), et = t + cT * Du1 * kTA, y = D2l * Dd1 * cB * D1r * kTA;
   off[0] = 0;
   off[1] = t;
   off[2] = et > y ? et : y;
-  off[3] = off[2] + a.D1l * a.Du1 * pad4(a.D1r * a.Dd1);
-  off[4] = off[3] + a.D2l * a.Dd1 * pad4(a.D2r * a.Dd2);
-  off[5] = off[4] + a.cB * a.Dd2 * pad4(a.cB2);
+  off[3] = off[2] + D1l * Du1 * pad4(D1r * Dd1);
+  off[4] = off[3] + D2l * Dd1 * pad4(D2r * Dd2);
+  off[5] = off[4] + cB * Dd2 * pad4(cB2);
   off[6] = off[5] + (several || x > z ? x : z);
   return off[6] + (several ? z : 0);
 }
@@ -368,9 +378,15 @@ cudaError_t allow_smem(K kernel) {
 
 }  // namespace
 
+// The kernels address an operand's tile by 32-bit offsets.  What lies in shared memory as a whole
+// bounds them; of T only a tile does, so its extent is looked at by itself.
+static bool tile_in_32_bits(int cT, long long sTa, int Du, long long sTu, long long sTa2) {
+  return (double)(cT - 1) * sTa + (double)(Du - 1) * sTu + (double)(kTA - 1) * sTa2 <= INT_MAX;
+}
+
 bool env3_f32_fits(const Env3Fused& a) {
-  int off[5];
-  return (long long)layout3(a, off) * 4 <= kMaxSmem;
+  double off[5];
+  return layout3(a, off) * 4 <= kMaxSmem && tile_in_32_bits(a.cT, a.sTa, a.Du, a.sTu, a.sTa2);
 }
 
 cudaError_t env3_f32(const Env3Fused& a, float* out1, bool rev2, bool rev3, const Mid3& mid, cudaStream_t st) {
@@ -390,8 +406,9 @@ cudaError_t env3_f32(const Env3Fused& a, float* out1, bool rev2, bool rev3, cons
 static bool several(const Env4Outs& o) { return (o.p[0] != nullptr) + (o.p[1] != nullptr) + (o.p[2] != nullptr) + (o.p[3] != nullptr) > 1; }
 
 bool env4_f32_fits(const Env4Fused& a, const Env4Outs& outs) {
-  int off[7];
-  return a.sEl1 == (long long)a.D2l * a.sEl2 && (long long)layout4(a, several(outs), off) * 4 <= kMaxSmem;
+  double off[7];
+  return a.sEl1 == (long long)a.D2l * a.sEl2 && layout4(a, several(outs), off) * 4 <= kMaxSmem &&
+         tile_in_32_bits(a.cT, a.sTa, a.Du1, a.sTu, a.sTa2);
 }
 
 cudaError_t env4_f32(const Env4Fused& a, const Env4Outs& outs, bool rev, cudaStream_t st) {

@@ -1,0 +1,181 @@
+// A CUDA runtime of the host alone, for tests of the launching code on a machine without a GPU:
+// linked with the library's objects in the place of libcudart.  Kernels do not run; every launch
+// is recorded under its kernel's name.  A launch that asks for more than 48 KB of dynamic shared
+// memory is refused unless that kernel's limit was raised on the current device since that device
+// was last reset, and errors stay pending until cudaGetLastError, as the runtime documents.
+#include <cuda_runtime_api.h>
+#include <stdint.h>
+#include <string.h>
+
+#include <map>
+#include <string>
+#include <utility>
+#include <vector>
+
+#include "fused.cuh"
+#include "fused_f32.cuh"
+#include "stages.cuh"
+
+namespace {
+
+struct Launch {
+  std::string name;
+  dim3 grid, block;
+  size_t smem;
+  bool early;
+};
+std::map<const void*, std::string> names;
+std::map<std::pair<int, const void*>, size_t> limits;  // dynamic shared memory, by device and kernel
+std::vector<Launch> launches;
+cudaError_t pending = cudaSuccess;
+int device = 0, refuse_limits = 0;
+bool capture_elsewhere = false;
+
+cudaError_t set(cudaError_t e) {
+  if (e != cudaSuccess) pending = e;
+  return e;
+}
+cudaError_t launch(const void* f, dim3 g, dim3 b, size_t smem, bool early) {
+  if (capture_elsewhere) return set(cudaErrorStreamCaptureImplicit);
+  const auto l = limits.find({device, f});
+  if (smem > (l == limits.end() ? 48u * 1024u : l->second)) return set(cudaErrorInvalidValue);
+  if (!g.x || g.x > 0x7fffffffu || g.y > 65535u || g.z > 65535u) return set(cudaErrorInvalidConfiguration);
+  launches.push_back(Launch{names[f], g, b, smem, early});
+  return cudaSuccess;
+}
+struct {
+  dim3 g, b;
+  size_t smem;
+  void* st;
+} config;
+
+}  // namespace
+
+extern "C" {
+
+void** __cudaRegisterFatBinary(void*) {
+  static void* handle;
+  return &handle;
+}
+void __cudaRegisterFatBinaryEnd(void**) {}
+void __cudaUnregisterFatBinary(void**) {}
+void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
+void __cudaRegisterFunction(void**, const char* f, char*, const char* name, int, uint3*, uint3*, dim3*, dim3*, int*) {
+  names[f] = name;
+}
+unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t smem, struct CUstream_st* st) {
+  config = {g, b, smem, st};
+  return 0;
+}
+cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* smem, void* st) {
+  *g = config.g;
+  *b = config.b;
+  *smem = config.smem;
+  memcpy(st, &config.st, sizeof(void*));
+  return cudaSuccess;
+}
+cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) {
+  *k = (cudaKernel_t)f;
+  return cudaSuccess;
+}
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void**, size_t smem, cudaStream_t) {
+  return launch((const void*)k, g, b, smem, false);
+}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
+  bool early = false;
+  for (unsigned i = 0; i < c->numAttrs; ++i) early |= c->attrs[i].id == cudaLaunchAttributeProgrammaticStreamSerialization;
+  return launch(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, early);
+}
+cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
+  if (refuse_limits > 0) {
+    --refuse_limits;
+    return set(cudaErrorNotReady);
+  }
+  if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) limits[{device, f}] = (size_t)v;
+  return cudaSuccess;
+}
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
+  if (capture_elsewhere) return set(cudaErrorStreamCaptureImplicit);
+  *s = cudaStreamCaptureStatusNone;
+  return cudaSuccess;
+}
+cudaError_t cudaGetLastError() {
+  const cudaError_t e = pending;
+  pending = cudaSuccess;
+  return e;
+}
+cudaError_t cudaPeekAtLastError() { return pending; }
+cudaError_t cudaGetDevice(int* d) {
+  *d = device;
+  return cudaSuccess;
+}
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int d) {
+  *v = a == cudaDevAttrMultiProcessorCount ? (d ? 76 : 152) : 0;
+  return cudaSuccess;
+}
+cudaError_t cudaGetSymbolAddress(void** p, const void* s) {
+  *p = const_cast<void*>(s);
+  return cudaSuccess;
+}
+const char* cudaGetErrorString(cudaError_t) { return "error of the fake runtime"; }
+
+// What the tests here do not reach.
+#define UNUSED(name, ...) \
+  cudaError_t name(__VA_ARGS__) { return set(cudaErrorNotSupported); }
+UNUSED(cudaDeviceSynchronize)
+UNUSED(cudaEventCreate, cudaEvent_t*)
+UNUSED(cudaEventCreateWithFlags, cudaEvent_t*, unsigned)
+UNUSED(cudaEventDestroy, cudaEvent_t)
+UNUSED(cudaEventElapsedTime, float*, cudaEvent_t, cudaEvent_t)
+UNUSED(cudaEventRecord, cudaEvent_t, cudaStream_t)
+UNUSED(cudaEventSynchronize, cudaEvent_t)
+UNUSED(cudaFree, void*)
+UNUSED(cudaGraphDestroy, cudaGraph_t)
+UNUSED(cudaGraphExecDestroy, cudaGraphExec_t)
+UNUSED(cudaGraphInstantiate, cudaGraphExec_t*, cudaGraph_t, unsigned long long)
+UNUSED(cudaGraphLaunch, cudaGraphExec_t, cudaStream_t)
+UNUSED(cudaMalloc, void**, size_t)
+UNUSED(cudaMemcpyAsync, void*, const void*, size_t, cudaMemcpyKind, cudaStream_t)
+UNUSED(cudaMemsetAsync, void*, int, size_t, cudaStream_t)
+UNUSED(cudaStreamBeginCapture, cudaStream_t, cudaStreamCaptureMode)
+UNUSED(cudaStreamCreateWithFlags, cudaStream_t*, unsigned)
+UNUSED(cudaStreamDestroy, cudaStream_t)
+UNUSED(cudaStreamEndCapture, cudaStream_t, cudaGraph_t*)
+UNUSED(cudaStreamSynchronize, cudaStream_t)
+UNUSED(cudaStreamWaitEvent, cudaStream_t, cudaEvent_t, unsigned)
+
+// ---- what the tests set and read
+void fake_device(int d) { device = d; }
+void fake_reset_device() {
+  for (auto it = limits.begin(); it != limits.end();) it = it->first.first == device ? limits.erase(it) : ++it;
+}
+void fake_refuse_limits(int n) { refuse_limits = n; }
+void fake_capture_elsewhere(int on) { capture_elsewhere = on; }
+void fake_pending(int e) { pending = (cudaError_t)e; }
+int fake_launches() { return (int)launches.size(); }
+void fake_clear() { launches.clear(); }
+const char* fake_name(int i) { return launches[i].name.c_str(); }
+long long fake_grid(int i) { return (long long)launches[i].grid.x * launches[i].grid.y * launches[i].grid.z; }
+long long fake_smem(int i) { return (long long)launches[i].smem; }
+
+// ---- the library's launchers by plain arguments; d: bonds and legs in the order of the C ABI
+int host_env3_f32_fits(int n, const int* d) {
+  pv::Env3Fused f;
+  f.batch = n;
+  f.cT = d[0]; f.cB = d[1]; f.cT2 = d[2]; f.cB2 = d[3]; f.Dl = d[4]; f.Dr = d[5]; f.Du = d[6]; f.Dd = d[7];
+  f.sTa = (long long)f.Du * f.cT2; f.sTu = f.cT2; f.sTa2 = 1;
+  return pv::env3_f32_fits(f);
+}
+int host_env4_f32_fits(int n, const int* d, int variants) {
+  pv::Env4Fused f;
+  f.batch = n;
+  f.cT = d[0]; f.cB = d[1]; f.cT2 = d[2]; f.cB2 = d[3];
+  f.D1l = d[4]; f.D1r = d[5]; f.Du1 = d[6]; f.Dd1 = d[7]; f.D2l = d[8]; f.D2r = d[9]; f.Dd2 = d[10];
+  f.sEl2 = f.cB; f.sEl1 = (long long)f.D2l * f.cB;
+  f.sTa = (long long)f.Du1 * f.cT2; f.sTu = f.cT2; f.sTa2 = 1;
+  pv::Env4Outs o;
+  for (int i = 0; i < variants; ++i) o.p[i] = (float*)16;
+  return pv::env4_f32_fits(f, o);
+}
+
+}  // extern "C"
