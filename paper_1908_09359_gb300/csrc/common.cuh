@@ -70,6 +70,30 @@ enum : unsigned {
   ST_TIMEOUT = 4u,
 };
 
+// Both of the following hold for the device and context that are current when a launch is made, so
+// they are asked for at every launch and nothing is kept: a process may use several devices, or
+// reset one.  (0.2 us and 0.03 us of host time, where a launch takes 1.5.)
+//
+// A kernel may have more than 48 KB of shared memory, its static variables included, only once its
+// limit of dynamic shared memory is raised.  bytes: the most that any launch of this kernel asks
+// for, so that threads that launch it with different sizes do not lower each other's limit.  all: the SM's whole shared memory rather than
+// first-level cache, so that as many CTAs as planned fit an SM.
+constexpr size_t kCtaSmem = 227 * 1024;  // what a CTA of sm_103a may have, static and dynamic
+template <typename... Par>
+cudaError_t allow_smem(void (*kernel)(Par...), size_t bytes, bool all = false) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess && all) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  if (e != cudaSuccess) cudaGetLastError();  // reported here, so not once more by the next launch's check
+  return e;
+}
+inline cudaError_t sm_count(int* sms) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
 // Launch that may begin when the blocks of the kernel ahead of it on the stream have ended, before
 // its end is complete (programmatic dependent launch).  A call is hundreds to thousands of
 // dependent launches of a few us: launched one by one, a 4x4 measurement took 1.86 ms with

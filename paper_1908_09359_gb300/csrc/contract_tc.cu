@@ -291,12 +291,7 @@ template <int EB, int BN, bool X3, bool DB = false>
 cudaError_t launch(const GemmDesc& d, unsigned* status, cudaStream_t st) {
   // two plain stages, one split stage, or two split stages (DB)
   constexpr int smem = (DB ? 4 : 2) * (kBM + BN) * kKBytes;
-  static bool configured = false;
-  if (!configured) {
-    PV_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EB, BN, X3, DB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 smem));
-    configured = true;
-  }
+  PV_CUDA(allow_smem(gemm_tc_kernel<EB, BN, X3, DB>, smem));
   const int tiles = ((d.M + kBM - 1) / kBM) * ((d.N + BN - 1) / BN);
   dim3 grid(tiles, d.batch < 65535 ? d.batch : 65535, (d.batch + 65534) / 65535);
   return launch_early(gemm_tc_kernel<EB, BN, X3, DB>, grid, kThreads, smem, st, d, status);

@@ -416,23 +416,9 @@ __global__ void __launch_bounds__(kPipeThreads, 1) env3_fused_kernel(const __gri
   if (warp == 0) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-template <typename K>
-cudaError_t configure(K kernel, uint32_t smem) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-int sm_count() {
-  static const int sms = [] {
-    int dev = 0, n = 0;
-    return cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess
-               ? n : 1;
-  }();
-  return sms;
-}
-
 template <bool X3, bool FULL>
 cudaError_t launch(const Plan3& P, int grid, unsigned* status, cudaStream_t st) {
-  static const cudaError_t configured = configure(env3_fused_kernel<X3, FULL>, SMEM_BYTES);
-  PV_CUDA(configured);
+  PV_CUDA(allow_smem(env3_fused_kernel<X3, FULL>, SMEM_BYTES));
   return launch_early(env3_fused_kernel<X3, FULL>, grid, kPipeThreads, SMEM_BYTES, st, P, status);
 }
 
@@ -727,8 +713,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) proj3_fused_kernel(const __gr
 
 template <bool X3, bool FULL>
 cudaError_t launch_proj3(const PlanP& P, int grid, unsigned* status, cudaStream_t st) {
-  static const cudaError_t configured = configure(proj3_fused_kernel<X3, FULL>, P_SMEM_BYTES);
-  PV_CUDA(configured);
+  PV_CUDA(allow_smem(proj3_fused_kernel<X3, FULL>, P_SMEM_BYTES));
   return launch_early(proj3_fused_kernel<X3, FULL>, grid, kPipeThreads, P_SMEM_BYTES, st, P, status);
 }
 
@@ -744,8 +729,9 @@ cudaError_t env3_fused(const Env3Fused& a, bool split, unsigned* status, cudaStr
   if (g_dry_run || a.batch <= 0) return cudaSuccess;
   if (!env3_fused_fits(a.cT, a.cB, a.cT2, a.cB2, a.Dl, a.Dr, a.Du, a.Dd)) return cudaErrorInvalidValue;
   if ((long long)a.batch * 4 > 0x7fffffffLL) return cudaErrorInvalidValue;
-  int grid = 0;
-  const Plan3 P = plan3(a, sm_count(), grid);
+  int grid = 0, sms = 0;
+  PV_CUDA(sm_count(&sms));
+  const Plan3 P = plan3(a, sms, grid);
   const bool full = all_full(P.op);
   // One a' tile per chain leaves a stream idle, and few tiles leave nothing to overlap: one
   // tile per CTA is then faster.  Tiles (a' x b) of a launch, one tile per CTA / pipeline,
@@ -761,8 +747,9 @@ cudaError_t proj3_fused(const Proj3Fused& a, bool split, unsigned* status, cudaS
   if (g_dry_run || a.batch <= 0) return cudaSuccess;
   if (!proj3_fused_fits(a)) return cudaErrorInvalidValue;
   if ((long long)a.batch * 2 > 0x7fffffffLL) return cudaErrorInvalidValue;
-  int grid = 0;
-  const PlanP P = planp(a, sm_count(), grid);
+  int grid = 0, sms = 0;
+  PV_CUDA(sm_count(&sms));
+  const PlanP P = planp(a, sms, grid);
   // With one or two a' tiles there is too little per unit to overlap.  Measured, one tile per
   // CTA / pipeline, split BF16: full bonds 16 chains 22.5 / 18.3 us, 512 chains 98.8 / 66.9;
   // Dc 16, D 4 (two a' tiles) 64 chains 14.3 / 14.3, 512 chains 32.0 / 33.2.

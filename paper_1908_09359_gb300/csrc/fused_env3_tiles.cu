@@ -416,17 +416,10 @@ __global__ void __launch_bounds__(kThreads, 2) env3_tile_kernel(const Env3Fused 
 
 template <bool X3>
 cudaError_t launch(const Env3Fused& a, unsigned* status, cudaStream_t st) {
-  static int ctas = 0;
-  if (!ctas) {
-    PV_CUDA(cudaFuncSetAttribute(env3_tile_kernel<X3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)SMEM_BYTES));
-    // the whole shared memory for this kernel, so that two CTAs fit an SM
-    PV_CUDA(cudaFuncSetAttribute(env3_tile_kernel<X3>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    int dev = 0, sms = 0;
-    PV_CUDA(cudaGetDevice(&dev));
-    PV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    ctas = 2 * sms;  // two resident CTAs per SM (104 KB shared memory, 128 registers x 256 threads each)
-  }
+  PV_CUDA(allow_smem(env3_tile_kernel<X3>, SMEM_BYTES, true));
+  int sms = 0;
+  PV_CUDA(sm_count(&sms));
+  const int ctas = 2 * sms;  // two resident CTAs per SM (104 KB shared memory, 128 registers x 256 threads each)
   const long long units = (long long)a.batch * ((a.cT2 + kAT - 1) / kAT);
   if (units > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = (int)(units < ctas ? units : ctas);
@@ -707,16 +700,10 @@ __global__ void __launch_bounds__(kThreads, 2) proj3_tile_kernel(const Proj3Fuse
 
 template <bool X3>
 cudaError_t launch_proj3(const Proj3Fused& a, unsigned* status, cudaStream_t st) {
-  static int ctas = 0;
-  if (!ctas) {
-    PV_CUDA(cudaFuncSetAttribute(proj3_tile_kernel<X3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)P_SMEM_BYTES));
-    PV_CUDA(cudaFuncSetAttribute(proj3_tile_kernel<X3>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    int dev = 0, sms = 0;
-    PV_CUDA(cudaGetDevice(&dev));
-    PV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    ctas = 2 * sms;
-  }
+  PV_CUDA(allow_smem(proj3_tile_kernel<X3>, P_SMEM_BYTES, true));
+  int sms = 0;
+  PV_CUDA(sm_count(&sms));
+  const int ctas = 2 * sms;
   const long long units = (long long)a.batch * ((a.cV + kPV - 1) / kPV);
   if (units > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = (int)(units < ctas ? units : ctas);

@@ -459,9 +459,7 @@ void set_site(PipeOp& o, const float* base, long long slot, int nl, long long sl
 
 template <bool X3>
 cudaError_t launch(const Plan4& P, int grid, unsigned* status, cudaStream_t st) {
-  static const cudaError_t configured =
-      cudaFuncSetAttribute(env4_pipe_kernel<X3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-  PV_CUDA(configured);
+  PV_CUDA(allow_smem(env4_pipe_kernel<X3>, SMEM_BYTES));
   return launch_early(env4_pipe_kernel<X3>, grid, kThreads, SMEM_BYTES, st, P, status);
 }
 
@@ -483,11 +481,8 @@ bool env4_pipe_fits(const Env4Fused& a, void* plan) {
 
 cudaError_t env4_pipe(const void* plan, bool split, unsigned* status, cudaStream_t st) {
   Plan4 P = *static_cast<const Plan4*>(plan);
-  static const int sms = [] {
-    int dev = 0, n = 0;
-    return cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess
-               ? n : 1;
-  }();
+  int sms = 0;
+  PV_CUDA(sm_count(&sms));
   const int units = 4 * P.a.batch, grid = units < sms ? units : sms;
   P.share = units / grid;
   P.rest = units % grid;

@@ -37,7 +37,7 @@ namespace pv {
 namespace {
 
 constexpr int kTA = 8;        // a' per CTA
-constexpr int kMaxSmem = 227 * 1024 - 1024;
+constexpr int kMaxSmem = kCtaSmem - 1024;
 
 // One product of the chain.  Operand P (rows): element (k, i, j) at p + k*ldp + i*8 + j; operand
 // Q (columns): element (k, c) at q + k*ldq + c (ldq and c padded to 4).  Output (i, c, j) at
@@ -371,11 +371,6 @@ int threads_for(int tasks, int smem) {
   return tasks > 256 && 2 * (smem + 1024) > 228 * 1024 ? 512 : tasks > 128 ? 256 : tasks > 64 ? 128 : 64;
 }
 
-template <typename K>
-cudaError_t allow_smem(K kernel) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-}
-
 }  // namespace
 
 // The kernels address an operand's tile by 32-bit offsets.  What lies in shared memory as a whole
@@ -393,13 +388,11 @@ cudaError_t env3_f32(const Env3Fused& a, float* out1, bool rev2, bool rev3, cons
   if (g_dry_run || a.batch <= 0) return cudaSuccess;
   int off[5];
   const int smem = layout3(a, off) * 4;
-  static const cudaError_t allowed = allow_smem(env3_f32_kernel<false>), allowed_mid = allow_smem(env3_f32_kernel<true>);
-  PV_CUDA(allowed);
-  PV_CUDA(allowed_mid);
   const long long blocks = (long long)a.batch * ((a.cT2 + kTA - 1) / kTA);
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int tasks = a.Du * ((a.Dl * a.cB + 3) / 4), tasks2 = a.cB * ((a.Dr * a.Dd + 3) / 4);
   auto* kernel = mid.p ? env3_f32_kernel<true> : env3_f32_kernel<false>;
+  if (smem > 48 * 1024) PV_CUDA(allow_smem(kernel, kMaxSmem));
   return launch_early(kernel, (unsigned)blocks, threads_for(tasks > tasks2 ? tasks : tasks2, smem), smem, st, a, out1, rev2, rev3, mid);
 }
 
@@ -415,8 +408,7 @@ cudaError_t env4_f32(const Env4Fused& a, const Env4Outs& outs, bool rev, cudaStr
   if (g_dry_run || a.batch <= 0) return cudaSuccess;
   int off[7];
   const int smem = layout4(a, several(outs), off) * 4;
-  static const cudaError_t allowed = allow_smem(env4_f32_kernel);
-  PV_CUDA(allowed);
+  if (smem > 48 * 1024) PV_CUDA(allow_smem(env4_f32_kernel, kMaxSmem));
   const long long blocks = (long long)a.batch * ((a.cT2 + kTA - 1) / kTA);
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int tasks = a.D2l * a.cB * ((a.D1r * a.Dd1 + 3) / 4);

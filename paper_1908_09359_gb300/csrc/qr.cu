@@ -435,11 +435,9 @@ cudaError_t qr_pos_batched(const float* Y, long long bsY, long long yrs, long lo
     return launch_tree<2, 4>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols, batch, st);
   }
   const size_t smem = (size_t)2 * rows * cols * sizeof(float);
-  static size_t configured = 0;
-  if (smem > 48 * 1024 && smem > configured) {
-    PV_CUDA(cudaFuncSetAttribute(qr_pos_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    configured = smem;
-  }
+  constexpr size_t kMost = kCtaSmem - kQrMaxCols * (sizeof(float) + sizeof(int)) - kQrThreads / 32 * sizeof(float);
+  if (smem > kMost) return cudaErrorInvalidValue;
+  PV_CUDA(allow_smem(qr_pos_kernel, kMost));
   qr_pos_kernel<<<batch, kQrThreads, smem, st>>>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols);
   return cudaGetLastError();
 }

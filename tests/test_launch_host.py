@@ -32,7 +32,9 @@ def fake(tmp_path_factory):
 
 @pytest.fixture(autouse=True)
 def clean(fake):
-    fake.fake_device(0)
+    for d in (1, 0):
+        fake.fake_device(d)
+        fake.fake_reset_device()
     fake.fake_refuse_limits(0)
     fake.fake_capture_elsewhere(0)
     fake.fake_pending(0)
@@ -86,3 +88,61 @@ def test_fp32_three_line_step_is_fused_only_where_it_fits(fake, n, dims, fused):
 ])
 def test_fp32_four_line_step_is_fused_only_where_it_fits(fake, dims, variants, fits):
     assert fake.host_env4_f32_fits(1, (C.c_int * 11)(*dims), variants) == fits
+
+
+# Every kernel that takes more than 48 KB of shared memory, by a launcher that reaches it
+# (precision of the tensor-core launchers: 3 is split BF16, 2 BF16).
+BIG = {
+    "noalloc, Dc 24, D 6": (lambda f: noalloc(f, 8, (24, 24, 24, 24, 6, 6, 6, 6)), "env3_f32_kernel"),
+    "FP32 optimal site": (lambda f: f.host_proj_f32(8), "env3_f32_kernel"),
+    "FP32 four-line step": (lambda f: f.host_env4_f32(8), "env4_f32_kernel"),
+    "QR, 320 x 40": (lambda f: f.pepsvmc_qr_pos(E, OUT, 5, 320, 40, 0, None), "qr_pos_kernel"),
+    "three-line pipeline": (lambda f: f.host_env3(512, 32, 8, 3), "env3_fused_kernel"),
+    "three-line pipeline, other bonds": (lambda f: f.host_env3(900, 24, 6, 2), "env3_fused_kernel"),
+    "three-line tiles": (lambda f: f.host_env3(8, 32, 8, 3), "env3_tile_kernel"),
+    "optimal-site pipeline": (lambda f: f.host_proj3(64, 32, 8, 3), "proj3_fused_kernel"),
+    "optimal-site tiles": (lambda f: f.host_proj3(64, 16, 4, 2), "proj3_tile_kernel"),
+    "four-line pipeline": (lambda f: f.host_env4(16, 32, 8, 3), "env4_pipe_kernel"),
+    "four-line tiles": (lambda f: f.host_env4(16, 24, 6, 3), "env4_fused_kernel"),
+    "QR, 304 x 20 (48 KB with its static variables)": (lambda f: f.pepsvmc_qr_pos(E, OUT, 5, 304, 20, 0, None), "qr_pos_kernel"),
+    "separate product, 64 columns (48 KB and static variables)": (lambda f: f.host_gemm_tc(3, 64), "gemm_tc_kernel"),
+    "separate product, 128 columns": (lambda f: f.host_gemm_tc(3, 128), "gemm_tc_kernel"),
+}
+
+
+@pytest.mark.parametrize("what", list(BIG))
+def test_shared_memory_is_granted_on_whatever_device_is_current(fake, what):
+    call, kernel = BIG[what]
+    grids = []
+
+    def runs():
+        assert call(fake) == OK
+        assert fake.fake_launches() == 1 and kernel in fake.fake_name(0).decode() and fake.fake_smem(0) > 47 * 1024
+        grids.append(fake.fake_grid(0))
+        fake.fake_clear()
+
+    runs()
+    fake.fake_device(1)         # another device, with half the SMs
+    runs()
+    assert grids[1] <= grids[0]
+    fake.fake_reset_device()    # reset: its limits are gone
+    runs()
+    fake.fake_device(0)
+    fake.fake_reset_device()
+    fake.fake_refuse_limits(1)  # a refusal is reported, and not kept
+    assert call(fake) != OK and fake.fake_launches() == 0
+    runs()
+    assert grids == [grids[0], grids[1], grids[1], grids[0]]
+
+
+@pytest.mark.parametrize("chains,chi,D", [(512, 32, 8), (900, 24, 6)])
+def test_pipelines_have_one_cta_for_each_sm_of_the_current_device(fake, chains, chi, D):
+    for device, sms in ((0, 152), (1, 76)):
+        fake.fake_device(device)
+        assert fake.host_env3(chains, chi, D, 3) == OK and fake.fake_grid(fake.fake_launches() - 1) == sms
+
+
+@pytest.mark.parametrize("rows,ok", [(905, True), (906, False)])
+def test_qr_takes_what_a_cta_can_hold(fake, rows, ok):
+    assert (fake.pepsvmc_qr_pos(E, OUT, 1, rows, 32, 0, None) == OK) == ok
+    assert fake.fake_launches() == ok
