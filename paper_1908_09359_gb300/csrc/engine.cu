@@ -2131,7 +2131,8 @@ int pepsvmc_env3_left(pepsvmc_ctx* x, const float* E, const float* T, const floa
     f.sel_stride = 1;
     const long long no = n_chains * f.bsO;
     if (env3_f32_fits(f) && !overlaps(out, no, E, n_chains * f.bsE) && !overlaps(out, no, T, n_chains * f.bsT) &&
-        !overlaps(out, no, A, 2 * f.ssA)) {
+        !overlaps(out, no, A, 2 * f.ssA) && !overlaps(out, no, B, n_chains * f.bsB) &&
+        !overlaps(out, no, spins, n_chains)) {
       cudaError_t e = x->step3_f32(f, nullptr, false, n_chains, true);
       return e == cudaSuccess ? PEPSVMC_OK : x->fail_cuda(e);
     }
@@ -2195,7 +2196,9 @@ int pepsvmc_env4_left(pepsvmc_ctx* x, const float* E, const float* T, const floa
   const Env4Outs outs{{out}};
   const long long no = n_chains * f.bsO;
   if (x->f32_fused() && env4_f32_fits(f, outs) && !overlaps(out, no, E, n_chains * f.bsE) &&
-      !overlaps(out, no, T, n_chains * f.bsT) && !overlaps(out, no, A1, 2 * s1) && !overlaps(out, no, A2, 2 * s2)) {
+      !overlaps(out, no, T, n_chains * f.bsT) && !overlaps(out, no, A1, 2 * s1) && !overlaps(out, no, A2, 2 * s2) &&
+      !overlaps(out, no, B, n_chains * f.bsB) && !overlaps(out, no, spins1, n_chains) &&
+      !overlaps(out, no, spins2, n_chains)) {
     ++x->launches;
     cudaError_t e = env4_f32(f, outs, false, x->st);
     return e == cudaSuccess ? PEPSVMC_OK : x->fail_cuda(e);

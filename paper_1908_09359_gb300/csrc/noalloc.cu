@@ -56,7 +56,7 @@ extern "C" int pepsvmc_env3_left_noalloc(const float* E, const float* T, const f
   f.out = out; f.bsO = (long long)cT2 * Dr * cB2; f.sOa2 = (long long)Dr * cB2; f.sOr = cB2; f.sOb2 = 1;
   const long long no = n_chains * f.bsO;
   if (env3_f32_fits(f) && !overlaps(out, no, E, n_chains * f.bsE) && !overlaps(out, no, T, n_chains * f.bsT) &&
-      !overlaps(out, no, A, 2 * f.ssA))
+      !overlaps(out, no, A, 2 * f.ssA) && !overlaps(out, no, B, n_chains * f.bsB) && !overlaps(out, no, spins, n_chains))
     return env3_f32(f, nullptr, false, false, Mid3(), (cudaStream_t)stream) == cudaSuccess ? PEPSVMC_OK : PEPSVMC_ECUDA;
   float* scratch = nullptr;
   const int rc = scratch_on_current_device(&scratch);

@@ -49,10 +49,14 @@ inline long long env3_scratch(const Env3Dims& d) {
   return a > b ? a : b;
 }
 
-// Whether n floats at p and m floats at q share memory.  The separate products read E, T and A
-// before they write the result, the one-kernel steps do not: a caller whose result lies over
-// one of those gets the separate products.
-inline bool overlaps(const float* p, long long n, const float* q, long long m) { return p < q + m && q < p + n; }
+// Whether n entries at p and m entries at q share memory.  The separate products have read E, T, A
+// and the spins, and a chain of one tile its B, before they write the result; the one-kernel steps
+// have not (a chain's tiles run on several CTAs): a caller whose result lies over one of those
+// gets the separate products.
+template <typename P, typename Q>
+inline bool overlaps(const P* p, long long n, const Q* q, long long m) {
+  return q && (const void*)p < (const void*)(q + m) && (const void*)q < (const void*)(p + n);
+}
 
 inline bool env3_dims_ok(const Env3Dims& d) {
   return d.cT > 0 && d.cB > 0 && d.cT2 > 0 && d.cB2 > 0 && d.Dl > 0 && d.Dr > 0 && d.Du > 0 && d.Dd > 0;

@@ -78,6 +78,18 @@ def test_fp32_three_line_step_is_fused_only_where_it_fits(fake, n, dims, fused):
     assert fake.host_env3_f32_fits(n, (C.c_int * 8)(*dims)) == fused
 
 
+@pytest.mark.parametrize("over", ["E", "T", "A", "B", "end of B", "spins"])
+def test_result_over_an_input_takes_the_separate_products(fake, over):
+    """They read every input of a chain before that chain's result is written; a fused step of two
+    tiles of the outgoing bond does not."""
+    n, dims = 4, (16, 16, 16, 16, 4, 4, 4, 4)
+    at = {"E": E, "T": T, "A": A, "B": B, "end of B": C.c_void_p(B.value + 4 * (n * 16 * 4 * 16 - 1)),
+          "spins": C.c_void_p(SP.value - 4 * n * 16 * 4 * 16 + 1)}[over]
+    assert noalloc(fake, n, dims, out=at) == OK and launched(fake) == SEPARATE
+    beside = C.c_void_p(B.value + 4 * n * 16 * 4 * 16)
+    assert noalloc(fake, n, dims, out=beside, spins=None) == OK and launched(fake) == ["env3_f32_kernel"]
+
+
 @pytest.mark.parametrize("dims,variants,fits", [
     ((16, 16, 16, 16, 4, 4, 4, 4, 4, 4, 4), 1, 1),
     ((16, 16, 16, 16, 4, 4, 4, 4, 4, 4, 4), 4, 1),
