@@ -70,6 +70,14 @@ enum : unsigned {
   ST_TIMEOUT = 4u,
 };
 
+// e, a runtime call's result, to be returned to the caller: as the runtime's last error it would be
+// reported a second time, by the next check in this library or of the caller's.  An error that was
+// pending before stays.
+inline cudaError_t reported(cudaError_t e) {
+  if (e != cudaSuccess && cudaPeekAtLastError() == e) cudaGetLastError();
+  return e;
+}
+
 // Both of the following hold for the device and context that are current when a launch is made, so
 // they are asked for at every launch and nothing is kept: a process may use several devices, or
 // reset one.  (0.2 us and 0.03 us of host time, where a launch takes 1.5.)
@@ -83,15 +91,13 @@ template <typename... Par>
 cudaError_t allow_smem(void (*kernel)(Par...), size_t bytes, bool all = false) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e == cudaSuccess && all) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  if (e != cudaSuccess) cudaGetLastError();  // reported here, so not once more by the next launch's check
-  return e;
+  return reported(e);
 }
 inline cudaError_t sm_count(int* sms) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) cudaGetLastError();
-  return e;
+  return reported(e);
 }
 
 // Launch that may begin when the blocks of the kernel ahead of it on the stream have ended, before
@@ -106,9 +112,8 @@ inline cudaError_t sm_count(int* sms) {
 // plain form is as fast or faster (80.1 against 80.8 ms), so a capture gets that.
 inline bool plain_launches(cudaStream_t st) {
   cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
-  cudaGetLastError();  // a capture elsewhere bars the legacy stream: the launch itself reports that
-  return true;
+  // a capture elsewhere bars the legacy stream: the launch itself reports that
+  return reported(cudaStreamIsCapturing(st, &s)) != cudaSuccess || s != cudaStreamCaptureStatusNone;
 }
 template <typename... Par, typename... Arg>
 cudaError_t launch_early(void (*kernel)(Par...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Arg&... arg) {
@@ -122,7 +127,7 @@ cudaError_t launch_early(void (*kernel)(Par...), dim3 grid, dim3 block, size_t s
   cfg.stream = st;
   cfg.attrs = &at;
   cfg.numAttrs = plain_launches(st) ? 0 : 1;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Par>(arg)...);
+  return reported(cudaLaunchKernelEx(&cfg, kernel, static_cast<Par>(arg)...));
 }
 #ifdef __CUDACC__
 __device__ __forceinline__ void after_previous() {

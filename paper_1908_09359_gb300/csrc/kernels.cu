@@ -501,7 +501,7 @@ cudaError_t launch_chains(void (*one)(Par...), void (*cluster)(Par...), int n, i
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = plain_launches(st) ? 1 : 2;
-  return cudaLaunchKernelEx(&cfg, cluster, arg...);
+  return reported(cudaLaunchKernelEx(&cfg, cluster, arg...));
 }
 
 __global__ void eloc_diag_kernel(const int8_t* spins, int Ly, int Lx, double J1, double J2, double* eloc,

@@ -29,7 +29,7 @@ static __device__ __align__(256) float noalloc_scratch[PEPSVMC_NOALLOC_SCRATCH_F
 // Device address of noalloc_scratch in the current context.
 int scratch_on_current_device(float** out) {
   void* p = nullptr;
-  if (cudaGetSymbolAddress(&p, noalloc_scratch) != cudaSuccess || !p) return PEPSVMC_ECUDA;
+  if (reported(cudaGetSymbolAddress(&p, noalloc_scratch)) != cudaSuccess || !p) return PEPSVMC_ECUDA;
   *out = static_cast<float*>(p);
   return PEPSVMC_OK;
 }

@@ -14,6 +14,7 @@
 
 #include "fused.cuh"
 #include "fused_f32.cuh"
+#include "kernels.cuh"
 #include "stages.cuh"
 
 namespace {
@@ -245,6 +246,7 @@ int host_proj_f32(int n) {
   mid.p = at(7);
   return pv::env3_f32(env3(n, 24, 6), nullptr, true, false, mid, nullptr);
 }
+int host_dot(int n) { return pv::k_dot(at(1), n, at(2), n, n, (double*)at(3), 4, &status, nullptr); }
 int host_gemm_tc(int mode, int bn) {
   pv::GemmDesc g;
   g.M = g.N = g.K = 128;

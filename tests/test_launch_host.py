@@ -158,3 +158,22 @@ def test_pipelines_have_one_cta_for_each_sm_of_the_current_device(fake, chains, 
 def test_qr_takes_what_a_cta_can_hold(fake, rows, ok):
     assert (fake.pepsvmc_qr_pos(E, OUT, 1, rows, 32, 0, None) == OK) == ok
     assert fake.fake_launches() == ok
+
+
+@pytest.mark.parametrize("launch", ["one block per chain", "clusters", "step"])
+def test_a_refused_launch_is_reported_once(fake, launch):
+    call = {"one block per chain": lambda: fake.host_dot(100), "clusters": lambda: fake.host_dot(9000),
+            "step": lambda: noalloc(fake, 8, (16, 16, 16, 16, 4, 4, 4, 4))}[launch]
+    plain = lambda: fake.pepsvmc_qr_pos(E, OUT, 5, 320, 40, 0, None)  # noqa: E731
+    fake.fake_capture_elsewhere(1)   # the default stream refuses everything meanwhile
+    assert call() != OK
+    fake.fake_capture_elsewhere(0)
+    assert fake.cudaPeekAtLastError() == 0
+    assert call() == OK and plain() == OK
+
+
+def test_an_error_of_the_callers_stays_the_callers(fake):
+    """Pending from before the call: neither reported as the launch's nor dropped."""
+    fake.fake_pending(999)
+    assert fake.host_dot(100) == OK and noalloc(fake, 8, (24, 24, 24, 24, 6, 6, 6, 6)) == OK
+    assert fake.cudaPeekAtLastError() == 999
