@@ -106,7 +106,9 @@ inline cudaError_t sm_count(int* sms) {
 // plain launches and 1.18 ms with these, an 8x8 sweep of 16 chains 25.2 and 17.8 ms.  Every kernel launched
 // this way calls after_previous() in all threads before it touches memory that another kernel may
 // write or read, and before any return, so that its own end still implies the end of
-// everything ahead of it.  No kernel lets the next one start earlier: blocks of the next one
+// everything ahead of it, and reads such memory by plain, volatile or asynchronous loads: one that promises
+// that the memory does not change during the kernel (__ldg, const __restrict__) may be moved ahead of
+// the wait.  No kernel lets the next one start earlier: blocks of the next one
 // then gathered on the few SMs that were free and took longer (a step of 128 chains of 8x8, D 8:
 // 91 against 81 ms).  In a graph, whose launches follow each other without the host, the
 // plain form is as fast or faster (80.1 against 80.8 ms), so a capture gets that.
