@@ -53,19 +53,28 @@ __device__ __forceinline__ float block_max(float v, float* red) {
   return m;
 }
 
-// Reductions over one chain's array longer than one block's registers hold (four-line
-// environments: up to 65,536 entries) run on a cluster of 2 to 8 blocks, each with a
-// contiguous slice; partial results are exchanged through distributed shared memory.  One
-// block per chain left most of the chip's loads unused at ordinary chain numbers.  Measured
-// on the 24x24 workload (D 8, Dc 32, 128 chains; mean over a step's launches with ~6 us of event
-// time each): normalisation 10.5 -> 7.8 us, ratio 26.9 -> 15.9, closure 21.5 -> 14.8; a step 1257 ->
-// 1193 ms.  The number of blocks follows from n alone.
+// Normalisation of arrays longer than one block's registers hold (four-line environments: up to
+// 65,536 entries): on a cluster of up to 8 blocks each slice is read once into registers and written
+// back scaled; one block reads the array twice.  What is scaled and by what does not depend on
+// the choice.  w: entries of the chain with the arrays that are scaled along (n if none).  Clusters
+// pay while there are few chains (latency), and where slices fill their blocks' registers and the
+// second pass would go to device memory; beyond that, scheduling the clusters costs more than
+// the second pass, which hits the second-level cache.  Measured, one block (as it was before there
+// were clusters) / always clusters / this rule, in a graph: 36,864 entries, 64 chains 6.5 / 5.3 / 5.3
+// us, 512 chains 18.4 / 32.1 / 18.0; 65,536 entries, 64 chains 16.8 / 7.1 / 6.9, 512 chains 66.7 / 49.1 /
+// 47.8, 512 chains with two more arrays 163 / 117 / 108; 8,200 entries, 512 chains 6.6 / 9.8 / 6.5.
 constexpr int kMaxCluster = 8;
 constexpr int kBlockEntries = 8192;
-inline int cluster_for(int n) {
+int normalize_blocks(int n, long long w, int batch, int sms) {
   int c = 1;
   while (c < kMaxCluster && (long long)c * kBlockEntries < n) c *= 2;
-  return c;
+  if (c == 1 || 4LL * n <= 5 * kBlockEntries) return 1;
+  if (4LL * batch <= (w > 2LL * n ? 5LL : 2LL) * sms) return c;
+  if (8LL * n > 7LL * c * kBlockEntries) {
+    if (4.0 * batch * w >= 96e6) return c;
+    if (c >= 4 && 8LL * batch <= 7LL * sms) return 4;
+  }
+  return 1;
 }
 // this block's slice of n entries, in multiples of 4
 __device__ __forceinline__ int slice_of(int n, int blocks, int rank, int* len) {
@@ -97,24 +106,46 @@ __device__ __forceinline__ void dot2_step(float& hi, float& lo, float a, float b
   hi = s;
   lo = __fadd_rn(lo, __fadd_rn(err, e));
 }
-// this thread's part of sum_i x[i] y[i] (Dot2 in float32 pairs, returned in float64)
-__device__ __forceinline__ double part_dot(const float* x, const float* y, int n) {
+__device__ __forceinline__ void dot2_step(float& hi, float& lo, const float4& a, const float4& b) {
+  dot2_step(hi, lo, a.x, b.x);
+  dot2_step(hi, lo, a.y, b.y);
+  dot2_step(hi, lo, a.z, b.z);
+  dot2_step(hi, lo, a.w, b.w);
+}
+// this thread's part of sum_i x[i] y[i] (Dot2 in float32 pairs, returned in float64), U of its
+// entries in flight at a time; the order of the sum does not depend on U
+template <int U, typename T>
+__device__ __forceinline__ double part_dot_of(const T* x, const T* y, int n) {
   float hi = 0.f, lo = 0.f;
-  if (vec4_ok(x, y, n)) {
-    const float4* x4 = reinterpret_cast<const float4*>(x);
-    const float4* y4 = reinterpret_cast<const float4*>(y);
-#pragma unroll 4
-    for (int i = threadIdx.x; i < (n >> 2); i += blockDim.x) {
-      const float4 a = x4[i], b = y4[i];
-      dot2_step(hi, lo, a.x, b.x);
-      dot2_step(hi, lo, a.y, b.y);
-      dot2_step(hi, lo, a.z, b.z);
-      dot2_step(hi, lo, a.w, b.w);
+  int i = threadIdx.x;
+  for (; i + (U - 1) * (int)blockDim.x < n; i += U * blockDim.x) {
+    T a[U], b[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      a[k] = x[i + k * blockDim.x];
+      b[k] = y[i + k * blockDim.x];
     }
-  } else {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) dot2_step(hi, lo, x[i], y[i]);
+#pragma unroll
+    for (int k = 0; k < U; ++k) dot2_step(hi, lo, a[k], b[k]);
+  }
+  if (i < n) {
+    T a[U - 1], b[U - 1];
+#pragma unroll
+    for (int k = 0; k < U - 1; ++k)
+      if (i + k * (int)blockDim.x < n) {
+        a[k] = x[i + k * blockDim.x];
+        b[k] = y[i + k * blockDim.x];
+      }
+#pragma unroll
+    for (int k = 0; k < U - 1; ++k)
+      if (i + k * (int)blockDim.x < n) dot2_step(hi, lo, a[k], b[k]);
   }
   return (double)hi + (double)lo;
+}
+template <int U = 4>
+__device__ __forceinline__ double part_dot(const float* x, const float* y, int n) {
+  return vec4_ok(x, y, n) ? part_dot_of<U>(reinterpret_cast<const float4*>(x), reinterpret_cast<const float4*>(y), n >> 2)
+                          : part_dot_of<U>(x, y, n);
 }
 // this thread's part of max |x[i]|; *bad set when an entry is not finite
 __device__ __forceinline__ float part_maxabs(const float* x, int n, bool* bad) {
@@ -174,8 +205,8 @@ __global__ void gather_kernel(float* dst, const double* src, const int* map, lon
 
 // Scale x (and x2, x3 by the same factor) by 2^-e, e the exponent of max|x|.  Up to
 // kBlockEntries entries per block (every three-line environment of Dc <= 32, D <= 8 in one
-// block, every four-line one in a cluster) are read once into registers and written back
-// scaled; larger arrays take a second pass.
+// block, a four-line one in a cluster) are read once into registers and written back
+// scaled; larger arrays or slices take a second pass.
 constexpr int kNormRegF4 = kBlockEntries / 4 / kThreads;
 template <bool CLUSTER>
 __global__ void normalize_pow2_kernel(float* x, long long bs, int n, float* x2, long long bs2, int n2, float* x3,
@@ -419,62 +450,57 @@ __global__ void phi_combine_kernel(const double* logpsi, const int8_t* sign, con
   }
 }
 
-// sum_i x[i] y[i] of one chain on a block or (CLUSTER) a cluster; the sum on rank 0's thread 0
-template <bool CLUSTER>
-__device__ __forceinline__ double chain_dot(const float* x, const float* y, int n, int blocks, int rank) {
-  namespace cg = cooperative_groups;
+// sum_i x[i] y[i] of one chain, on thread 0 (in block_sum's order), by one block: float64 additions are slow
+// here, so they are as few as the tree needs.  A block is bound by the latency of its loads while
+// it has an SM to itself, by bandwidth when many share one: U = 8 entries (16 loads of 16 bytes) in
+// flight up to two blocks per SM, beyond that U = 2 and more blocks.  Measured in a graph, U as the
+// compiler chose / clusters of up to 8 blocks / this: 65,536 entries, 16 chains 15.0 / 6.6 / 6.9 us, 128
+// chains 15.6 / 15.0 / 7.3, 512 chains 50.3 / 58.9 / 41.0; 20,736 entries, 256 chains 8.1 / 12.8 / 5.7; 4,096
+// entries, 1024 chains 11.0 / - / 7.3.
+inline cudaError_t deep_loads(int batch, bool* deep) {
+  int sms = 0;
+  PV_CUDA(sm_count(&sms));
+  *deep = batch <= 2 * sms;
+  return cudaSuccess;
+}
+template <int U>
+__device__ __forceinline__ double chain_dot(const float* x, const float* y, int n) {
   __shared__ double red[kThreads / 32];
-  __shared__ double part;
-  int off = 0, len = n;
-  if constexpr (CLUSTER) off = slice_of(n, blocks, rank, &len);
-  double s = block_sum(part_dot(x + off, y + off, len), red);
-  if constexpr (CLUSTER) {
-    if (threadIdx.x == 0) part = s;
-    cg::this_cluster().sync();
-    if (rank == 0 && threadIdx.x == 0)
-      for (int i = 1; i < blocks; ++i) s += *cg::this_cluster().map_shared_rank(&part, i);
-    cg::this_cluster().sync();  // `part` has been read before any block ends
-  }
+  double v = part_dot<U>(x, y, n);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x == 0)
+    for (int i = 0; i < kThreads / 32; ++i) s += red[i];
   return s;
 }
-// chain of this block; its place in the chain's cluster
-template <bool CLUSTER>
-__device__ __forceinline__ int chain_of(int* blocks, int* rank) {
-  *blocks = 1;
-  *rank = 0;
-  if constexpr (CLUSTER) {
-    *blocks = cooperative_groups::this_cluster().num_blocks();
-    *rank = cooperative_groups::this_cluster().block_rank();
-  }
-  return blockIdx.x / *blocks;
-}
 
-template <bool CLUSTER>
+template <int U>
 __global__ void dot_kernel(const float* a, long long bsa, const float* bb, long long bsb, int n, double* out,
                            unsigned* status) {
   after_previous();
-  int blocks, rank;
-  const int b = chain_of<CLUSTER>(&blocks, &rank);
-  const double s = chain_dot<CLUSTER>(a + b * bsa, bb + b * bsb, n, blocks, rank);
-  if (threadIdx.x == 0 && rank == 0) {
+  const int b = blockIdx.x;
+  const double s = chain_dot<U>(a + b * bsa, bb + b * bsb, n);
+  if (threadIdx.x == 0) {
     out[b] = s;
     if (s == 0.0) atomicOr(status, ST_ZEROPSI);
     if (!isfinite(s)) atomicOr(status, ST_NONFINITE);
   }
 }
 
-template <bool CLUSTER>
+template <int U>
 __global__ void ratio_accum_kernel(const float* a, long long bsa, const float* bb, long long bsb, int n,
                                    const double* den, const int8_t* spins, long long spin_stride, int si, int sj,
                                    double halfJ, double* eloc, unsigned* status, float* rho_out, long long rho_stride,
                                    long long rho_idx) {
   after_previous();
-  int blocks, rank;
-  const int b = chain_of<CLUSTER>(&blocks, &rank);
+  const int b = blockIdx.x;
   const int8_t* sp = spins + b * spin_stride;
-  if (sp[si] == sp[sj]) return;  // no off-diagonal element for a parallel pair (the whole cluster)
-  const double s = chain_dot<CLUSTER>(a + b * bsa, bb + b * bsb, n, blocks, rank);
-  if (threadIdx.x == 0 && rank == 0) {
+  if (sp[si] == sp[sj]) return;  // no off-diagonal element for a parallel pair
+  const double s = chain_dot<U>(a + b * bsa, bb + b * bsb, n);
+  if (threadIdx.x == 0) {
     const double r = s / den[b];
     if (!isfinite(r)) atomicOr(status, ST_NONFINITE);
     eloc[b] += halfJ * r;
@@ -482,13 +508,10 @@ __global__ void ratio_accum_kernel(const float* a, long long bsa, const float* b
   }
 }
 
-// One block per chain, or a cluster of them.
+// One block per chain, or a cluster of c.
 template <typename... Par, typename... Arg>
-cudaError_t launch_chains(void (*one)(Par...), void (*cluster)(Par...), int n, int batch, cudaStream_t st, Arg... arg) {
-  const int c = cluster_for(n);
-  if (c == 1 || batch > 0x7fffffff / c) {
-    return launch_early(one, batch, kThreads, 0, st, arg...);
-  }
+cudaError_t launch_chains(void (*kernel)(Par...), int c, int batch, cudaStream_t st, Arg... arg) {
+  if (c == 1) return launch_early(kernel, batch, kThreads, 0, st, arg...);
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = c;
@@ -501,9 +524,8 @@ cudaError_t launch_chains(void (*one)(Par...), void (*cluster)(Par...), int n, i
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = plain_launches(st) ? 1 : 2;
-  return reported(cudaLaunchKernelEx(&cfg, cluster, arg...));
+  return reported(cudaLaunchKernelEx(&cfg, kernel, arg...));
 }
-
 __global__ void eloc_diag_kernel(const int8_t* spins, int Ly, int Lx, double J1, double J2, double* eloc,
                                  int batch) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -719,8 +741,11 @@ cudaError_t k_gather_f32(float* dst, const double* src, const int* map, long lon
 cudaError_t k_normalize_pow2(float* x, long long bs, int n, float* x2, long long bs2, int n2, float* x3,
                              long long bs3, int n3, int* exps, int batch, unsigned* status, cudaStream_t st) {
   if (g_dry_run) return cudaSuccess;
-  return launch_chains(normalize_pow2_kernel<false>, normalize_pow2_kernel<true>, n, batch, st, x, bs, n, x2, bs2, n2, x3, bs3,
-                       n3, exps, status);
+  int sms = 0;
+  PV_CUDA(sm_count(&sms));
+  const int c = normalize_blocks(n, (long long)n + n2 + n3, batch, sms);
+  return launch_chains(c == 1 ? normalize_pow2_kernel<false> : normalize_pow2_kernel<true>, c, batch, st, x, bs, n, x2, bs2, n2, x3,
+                       bs3, n3, exps, status);
 }
 cudaError_t k_mps_normalize(float* x, long long bs, int n, const int* exps, const double* log_in, double* log_out,
                             int batch, unsigned* status, cudaStream_t st) {
@@ -745,15 +770,21 @@ cudaError_t k_phi_combine(const double* logpsi, const int8_t* sign, const double
 cudaError_t k_dot(const float* a, long long bsa, const float* b, long long bsb, int n, double* out, int batch,
                   unsigned* status, cudaStream_t st) {
   if (g_dry_run) return cudaSuccess;
-  return launch_chains(dot_kernel<false>, dot_kernel<true>, n, batch, st, a, bsa, b, bsb, n, out, status);
+  bool deep = false;
+  PV_CUDA(deep_loads(batch, &deep));
+  auto* k = deep ? dot_kernel<8> : dot_kernel<2>;
+  return launch_early(k, batch, kThreads, 0, st, a, bsa, b, bsb, n, out, status);
 }
 cudaError_t k_ratio_accum(const float* a, long long bsa, const float* b, long long bsb, int n, const double* den,
                           const int8_t* spins, long long spin_stride, int si, int sj, double halfJ, double* eloc,
                           int batch, unsigned* status, cudaStream_t st, float* rho_out, long long rho_stride,
                           long long rho_idx) {
   if (g_dry_run) return cudaSuccess;
-  return launch_chains(ratio_accum_kernel<false>, ratio_accum_kernel<true>, n, batch, st, a, bsa, b, bsb, n, den, spins,
-                       spin_stride, si, sj, halfJ, eloc, status, rho_out, rho_stride, rho_idx);
+  bool deep = false;
+  PV_CUDA(deep_loads(batch, &deep));
+  auto* k = deep ? ratio_accum_kernel<8> : ratio_accum_kernel<2>;
+  return launch_early(k, batch, kThreads, 0, st, a, bsa, b, bsb, n, den, spins, spin_stride, si, sj, halfJ, eloc, status, rho_out,
+                      rho_stride, rho_idx);
 }
 cudaError_t k_eloc_diag(const int8_t* spins, int Ly, int Lx, double J1, double J2, double* eloc, int batch,
                         cudaStream_t st) {

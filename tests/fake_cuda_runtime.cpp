@@ -246,7 +246,11 @@ int host_proj_f32(int n) {
   mid.p = at(7);
   return pv::env3_f32(env3(n, 24, 6), nullptr, true, false, mid, nullptr);
 }
-int host_dot(int n) { return pv::k_dot(at(1), n, at(2), n, n, (double*)at(3), 4, &status, nullptr); }
+int host_dot(int n, int chains) { return pv::k_dot(at(1), n, at(2), n, n, (double*)at(3), chains, &status, nullptr); }
+int host_normalize(int n, int arrays, int chains) {
+  return pv::k_normalize_pow2(at(1), n, n, arrays > 1 ? at(2) : nullptr, n, arrays > 1 ? n : 0, arrays > 2 ? at(3) : nullptr, n,
+                              arrays > 2 ? n : 0, (int*)at(4), chains, &status, nullptr);
+}
 int host_gemm_tc(int mode, int bn) {
   pv::GemmDesc g;
   g.M = g.N = g.K = 128;

@@ -1,10 +1,10 @@
 """Power-of-two normalisation of arrays that take a cluster of blocks (over 8,192 entries): what
-one slice alone knows -- the largest entry, one that is not finite -- has to reach all of them.
+one slice alone knows -- the largest entry, one that is not finite -- has to reach all of them;
+with many chains one block takes the same arrays in two passes, with the same results.
 The kernel's launcher is called directly: through a measurement the status of a chain would come
 from smaller arrays before."""
 import ctypes as C
 
-import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -36,20 +36,20 @@ def normalize():
 
 # 8,193 and 9,000: two blocks; 34,596: eight; 65,537: over eight blocks' registers; 12,289 of stride 12,291:
 # no 16-byte access
+@pytest.mark.parametrize("chains", [9, 300])
 @pytest.mark.parametrize("n,stride", [(8192, 8192), (8193, 8196), (9000, 9000), (12289, 12291), (34596, 34596), (65536, 65536),
                                       (65537, 65540), (100000, 100000)])
-def test_largest_entry_of_any_slice_and_bad_ones(normalize, n, stride):
+def test_largest_entry_of_any_slice_and_bad_ones(normalize, n, stride, chains):
     import torch
     torch.cuda.synchronize()
     g = torch.Generator(device="cuda").manual_seed(n)
-    chains = 9
     X = torch.randn(chains, stride, generator=g, device="cuda")[:, :n]
     X *= 1e-3
     places = [0, 3, n // 8 - 1, n // 8, n // 2, n // 2 + 5, n - n // 8, n - 2, n - 1]
     for c, i in enumerate(places):
         X[c, i] = -7.5 * 2.0 ** (c - 4)
     Y = torch.randn(chains, n + 3, generator=g, device="cuda")
-    want_e = torch.tensor([np.frexp(7.5 * 2.0 ** (c - 4))[1] for c in range(chains)], device="cuda")
+    want_e = torch.frexp(X.abs().amax(1))[1]
     x, y, exps = X.clone(), Y.clone(), torch.full((chains,), 5, dtype=torch.int32, device="cuda")
     assert normalize(x, y, None, exps) == 0
     shift = exps - 5
@@ -57,7 +57,7 @@ def test_largest_entry_of_any_slice_and_bad_ones(normalize, n, stride):
     f = torch.ldexp(torch.ones(chains, device="cuda"), -shift)[:, None]
     assert torch.equal(x, X * f) and torch.equal(y, Y * f)  # exact: powers of two
     for bad, bit in ((float("nan"), NONFINITE), (float("inf"), NONFINITE), (float("-inf"), NONFINITE), (0.0, ZEROPSI)):
-        for i in places:
+        for i in places if chains == 9 else places[-1:]:
             x, y, exps = X.clone(), Y.clone(), torch.full((chains,), 5, dtype=torch.int32, device="cuda")
             if bit == ZEROPSI:
                 x[4] = 0.0

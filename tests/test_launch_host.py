@@ -162,7 +162,7 @@ def test_qr_takes_what_a_cta_can_hold(fake, rows, ok):
 
 @pytest.mark.parametrize("launch", ["one block per chain", "clusters", "step"])
 def test_a_refused_launch_is_reported_once(fake, launch):
-    call = {"one block per chain": lambda: fake.host_dot(100), "clusters": lambda: fake.host_dot(9000),
+    call = {"one block per chain": lambda: fake.host_dot(100, 4), "clusters": lambda: fake.host_normalize(65536, 1, 4),
             "step": lambda: noalloc(fake, 8, (16, 16, 16, 16, 4, 4, 4, 4))}[launch]
     plain = lambda: fake.pepsvmc_qr_pos(E, OUT, 5, 320, 40, 0, None)  # noqa: E731
     fake.fake_capture_elsewhere(1)   # the default stream refuses everything meanwhile
@@ -175,5 +175,18 @@ def test_a_refused_launch_is_reported_once(fake, launch):
 def test_an_error_of_the_callers_stays_the_callers(fake):
     """Pending from before the call: neither reported as the launch's nor dropped."""
     fake.fake_pending(999)
-    assert fake.host_dot(100) == OK and noalloc(fake, 8, (24, 24, 24, 24, 6, 6, 6, 6)) == OK
+    assert fake.host_dot(100, 4) == OK and noalloc(fake, 8, (24, 24, 24, 24, 6, 6, 6, 6)) == OK
     assert fake.cudaPeekAtLastError() == 999
+
+
+# (entries, arrays, chains): blocks per chain on 152 SMs
+@pytest.mark.parametrize("n,arrays,chains,blocks", [
+    (8192, 1, 1, 1), (8200, 1, 64, 1), (12000, 1, 76, 2), (12000, 1, 77, 1), (36864, 1, 64, 8), (36864, 1, 512, 1),
+    (65536, 1, 76, 8), (65536, 1, 128, 4), (65536, 1, 256, 1), (65536, 1, 512, 8), (65536, 3, 128, 8), (20736, 3, 190, 4),
+    (20736, 3, 191, 1), (100000, 1, 2048, 8),
+])
+def test_clusters_only_where_they_pay(fake, n, arrays, chains, blocks):
+    assert fake.host_normalize(n, arrays, chains) == OK
+    assert fake.fake_grid(0) == blocks * chains and fake.fake_name(0).decode().count("normalize_pow2") == 1
+    fake.fake_clear()
+    assert fake.host_dot(n, chains) == OK and fake.fake_grid(0) == chains  # one order of the sum, whatever the chains
