@@ -32,8 +32,8 @@
 // the same chain, so E, T, A and B are converted and kept once for both.  What is left beside
 // the drains' latency (~960 cycles each) is the change of chain, where the products wait for
 // the conversion of the next operands (~4,000 of 25,000 cycles a chain at Dc 32, D 8).
-// Launches of few tiles, where there is nothing to overlap, go to fused_env3_tiles.cu (one
-// tile per CTA, two CTAs per SM).
+// Launches of few tiles of bonds below the maxima, where there is nothing to overlap, go to
+// fused_env3_tiles.cu (one tile per CTA, two CTAs per SM).
 //
 // Dc 32, D 8, split BF16, one tile per CTA -> this form: three-line step 128 chains 29.2 ->
 // 21.1 us, 512 chains 90.9 -> 52.8 us, 2048 chains 364 -> 176 us (launched early, back to back,
@@ -43,6 +43,8 @@
 // eight warps and written out by the drains, 64.5 us; by two groups of four, 90 us; all of it
 // unrolled in line (115 KB of code, instruction fetch at 79 % of its rate), 75 us; one rolled
 // loop for all operand kinds, 76 us; results written by the converting warps, 68 us.
+#include <math.h>
+
 #include "fused.cuh"
 #include "fused_pipe.cuh"
 
@@ -106,7 +108,7 @@ struct Bars3 {
 // Units: (chain, a' tiles of `step` streams); a CTA owns a contiguous range of items of `align`
 // units, so consecutive units mostly share the chain and with it E, T, A and B.  Two streams
 // per unit, except when that would leave SMs without work: then every a' tile is a unit of
-// its own (first stream only; 17 chains of three tiles 14.8 us, with two streams 19.1).
+// its own (first stream only; full bonds, 38 chains 10.2 us, with two streams 12.7).
 // When the last unit of a chain has no tile for the second stream, an item is a whole chain.
 struct Plan3 {
   Env3Fused a;
@@ -723,6 +725,31 @@ bool all_full(const PipeOp (&op)[4]) {
   return true;
 }
 
+// Whether the pipeline is faster than one tile per CTA with bonds below the maxima (with full bonds it
+// is at every number of chains: 1 chain 10.3 / 9.7 us, one tile per CTA / pipeline, split BF16, 38
+// 10.8 / 10.2, 50 14.2 / 12.8, 512 90.9 / 52.8).  With one a' tile per chain a stream idles (Dc 8, D 2,
+// 1024 chains 29.2 / 43.5), and few tiles leave nothing to overlap.  Above that both forms run
+// in whole rounds of CTAs, so which is faster changes back and forth with the number of chains
+// (Dc 24, D 6, 152 chains 21.3 / 17.6, 184 25.9 / 30.3, 256 37.1 / 30.4, 2048 261 / 188; Dc 16, D 4 in
+// BF16 640 23.8 / 27.1): the rule compares estimates (us), fitted to 219 launches of bonds up to 32
+// and 8 and 150 to 2048 chains (rms error 4 % for one tile per CTA, 7 % for the pipeline).  One tile per
+// CTA: by rounds of two CTAs per SM and, if the last round needs one only, that.  Pipeline: by
+// a CTA's chains and tiles.  Of the 219, two sizes remain that the choice makes slower than one tile
+// per CTA by more than 3 %, by 7 and 11 %.
+bool pipeline_pays(const Plan3& P, int sms, bool split) {
+  const Env3Fused& a = P.a;
+  const long long tiles = (long long)a.batch * P.n_at;
+  if (P.n_at < 2 || tiles * P.n_bt * 152 < 1100LL * sms) return false;
+  const double rounds = (double)(tiles / (2 * sms)), last = (double)(tiles % (2 * sms)), n = P.n_bt;
+  const double whole = rounds + (last > sms), half = last > 0 && last <= sms;
+  const double units = (double)(P.share + (P.rest > 0)) * P.align, chains = ceil(units / P.per_chain);
+  const double v = 1e-4 * (a.cT * (a.Dl * a.cB + a.Du * a.cT2) + a.Dl * a.Du * a.Dr * a.Dd + a.cB * a.Dd * a.cB2);  // operands
+  const double per_tile = split ? 2.2 + whole * (3.4 + 3.85 * n + 0.76 * v) + half * (3.5 * n - 1.1)
+                                : 2.9 + whole * (2.2 + 2.65 * n + 0.84 * v) + half * (1.45 * n + 0.25);
+  const double pipe = split ? 4.7 + chains * (4.1 + 1.9 * v) + 1.8 * units * n : 4.9 + chains * (2.9 + 1.2 * v) + 1.35 * units * n;
+  return 1.03 * pipe < per_tile;
+}
+
 }  // namespace
 
 cudaError_t env3_fused(const Env3Fused& a, bool split, unsigned* status, cudaStream_t st) {
@@ -733,12 +760,7 @@ cudaError_t env3_fused(const Env3Fused& a, bool split, unsigned* status, cudaStr
   PV_CUDA(sm_count(&sms));
   const Plan3 P = plan3(a, sms, grid);
   const bool full = all_full(P.op);
-  // One a' tile per chain leaves a stream idle, and few tiles leave nothing to overlap: one
-  // tile per CTA is then faster.  Tiles (a' x b) of a launch, one tile per CTA / pipeline,
-  // split BF16: full bonds 256 13.0 / 12.7 us, 512 17.0 / 15.0, 1024 29.2 / 21.1, 4096 90.9 /
-  // 52.8; Dc 24, D 6 384 16.7 / 19.8, 1536 39.6 / 33.2, 6144 127 / 96.9; Dc 16, D 4 1024 31.0 /
-  // 33.5 (in a step), 2048 54.4 / 48.8; one a' tile: Dc 8, D 2, 1024 tiles 29.2 / 43.5.
-  if (P.n_at < 2 || (long long)a.batch * P.n_at * P.n_bt < (full ? 400 : 1100)) return env3_tiles(a, split, status, st);
+  if (!full && !pipeline_pays(P, sms, split)) return env3_tiles(a, split, status, st);
   if (full) return split ? launch<true, true>(P, grid, status, st) : launch<false, true>(P, grid, status, st);
   return split ? launch<true, false>(P, grid, status, st) : launch<false, false>(P, grid, status, st);
 }
@@ -753,7 +775,9 @@ cudaError_t proj3_fused(const Proj3Fused& a, bool split, unsigned* status, cudaS
   // With one or two a' tiles there is too little per unit to overlap.  Measured, one tile per
   // CTA / pipeline, split BF16: full bonds 16 chains 22.5 / 18.3 us, 512 chains 98.8 / 66.9;
   // Dc 16, D 4 (two a' tiles) 64 chains 14.3 / 14.3, 512 chains 32.0 / 33.2.
-  if (P.n_at < 3) return proj3_tiles(a, split, status, st);
+  // One tile of v leaves a stream idle, which costs where each chain would still have a CTA in the
+  // one round of two per SM: cV 12, 192 chains 20.0 / 22.4; 152 chains 18.9 / 15.3, 580 chains 30.2 / 28.6.
+  if (P.n_at < 3 || (P.n_vt == 1 && a.batch > sms && a.batch <= 2 * sms)) return proj3_tiles(a, split, status, st);
   if (all_full(P.op))
     return split ? launch_proj3<true, true>(P, grid, status, st) : launch_proj3<false, true>(P, grid, status, st);
   return split ? launch_proj3<true, false>(P, grid, status, st) : launch_proj3<false, false>(P, grid, status, st);

@@ -221,10 +221,11 @@ static pv::Env4Fused env4(int n, int chi, int D, bool bmajor) {
 }
 static unsigned status;
 int host_env3(int n, int chi, int D, int mode) { return pv::env3_fused(env3(n, chi, D), mode == 3, &status, nullptr); }
-int host_proj3(int n, int chi, int D, int mode) {
+int host_proj3(int n, int chi, int cV, int D, int mode) {
   pv::Proj3Fused f;
   f.batch = n;
-  f.cT = f.cV = f.cT2 = f.cV2 = chi;
+  f.cT = f.cT2 = f.cV2 = chi;
+  f.cV = cV;
   f.Dl = f.Dr = f.Du = f.Dd = D;
   f.L = at(1); f.T = at(2); f.A = at(3); f.R = at(5); f.out = at(6);
   f.bsL = f.bsT = f.bsR = f.bsO = (long long)chi * D * chi;

@@ -111,9 +111,9 @@ BIG = {
     "QR, 320 x 40": (lambda f: f.pepsvmc_qr_pos(E, OUT, 5, 320, 40, 0, None), "qr_pos_kernel"),
     "three-line pipeline": (lambda f: f.host_env3(512, 32, 8, 3), "env3_fused_kernel"),
     "three-line pipeline, other bonds": (lambda f: f.host_env3(900, 24, 6, 2), "env3_fused_kernel"),
-    "three-line tiles": (lambda f: f.host_env3(8, 32, 8, 3), "env3_tile_kernel"),
-    "optimal-site pipeline": (lambda f: f.host_proj3(64, 32, 8, 3), "proj3_fused_kernel"),
-    "optimal-site tiles": (lambda f: f.host_proj3(64, 16, 4, 2), "proj3_tile_kernel"),
+    "three-line tiles": (lambda f: f.host_env3(8, 24, 6, 3), "env3_tile_kernel"),
+    "optimal-site pipeline": (lambda f: f.host_proj3(64, 32, 32, 8, 3), "proj3_fused_kernel"),
+    "optimal-site tiles": (lambda f: f.host_proj3(64, 16, 16, 4, 2), "proj3_tile_kernel"),
     "four-line pipeline": (lambda f: f.host_env4(16, 32, 8, 3), "env4_pipe_kernel"),
     "four-line tiles": (lambda f: f.host_env4(16, 24, 6, 3), "env4_fused_kernel"),
     "QR, 304 x 20 (48 KB with its static variables)": (lambda f: f.pepsvmc_qr_pos(E, OUT, 5, 304, 20, 0, None), "qr_pos_kernel"),
@@ -190,3 +190,19 @@ def test_clusters_only_where_they_pay(fake, n, arrays, chains, blocks):
     assert fake.fake_grid(0) == blocks * chains and fake.fake_name(0).decode().count("normalize_pow2") == 1
     fake.fake_clear()
     assert fake.host_dot(n, chains) == OK and fake.fake_grid(0) == chains  # one order of the sum, whatever the chains
+
+
+@pytest.mark.parametrize("n,chi,D,mode,kernel", [
+    (1, 32, 8, 3, "fused"), (40, 32, 8, 2, "fused"), (512, 32, 8, 3, "fused"),
+    (60, 31, 8, 3, "tile"), (152, 24, 6, 3, "tile"), (184, 24, 6, 3, "tile"), (200, 20, 5, 3, "tile"), (256, 24, 6, 3, "fused"),
+    (640, 16, 4, 2, "tile"), (2048, 16, 4, 3, "fused"), (4096, 8, 2, 3, "tile"),
+])
+def test_three_line_step_takes_the_faster_form(fake, n, chi, D, mode, kernel):
+    """Measured on 152 SMs, one tile per CTA / pipeline: 184 chains of Dc 24, D 6 25.9 / 30.3 us, 640 of Dc 16,
+    D 4 in BF16 23.8 / 27.1; 256 of Dc 24, D 6 37.1 / 30.4, one of full bonds 10.3 / 9.7."""
+    assert fake.host_env3(n, chi, D, mode) == OK and f"env3_{kernel}_kernel" in fake.fake_name(0).decode()
+
+
+@pytest.mark.parametrize("n,cV,kernel", [(152, 12, "fused"), (192, 12, "tile"), (304, 16, "tile"), (305, 16, "fused"), (192, 17, "fused")])
+def test_optimal_site_takes_the_faster_form(fake, n, cV, kernel):
+    assert fake.host_proj3(n, 24, cV, 6, 3) == OK and f"proj3_{kernel}_kernel" in fake.fake_name(0).decode()
