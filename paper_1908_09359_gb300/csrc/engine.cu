@@ -998,7 +998,7 @@ struct pepsvmc_ctx {
       return fused4(fused4_left(E, bsE, cT, cB, T, bsT, cT2, a1, f1, a2, f2, B, bsB, cB2, out, bsO));
     const Env4Fused f = fused4_left(E, bsE, cT, cB, T, bsT, cT2, a1, f1, a2, f2, B, bsB, cB2, out, bsO);
     const Env4Outs o{{out}};
-    if (f32_fused() && env4_f32_fits(f, o)) return step4_f32(f, o, false);
+    if (f32_fused() && env4_f32_takes(f, o, C)) return step4_f32(f, o, false);
     PV_CUDA(left4_x(E, bsE, cT, cB, T, bsT, cT2, a1, a2, tmp1));
     PV_CUDA(left4_y(tmp1, cB, cT2, a1, f1, a2, tmp2));
     return left4_zw(tmp2, cB, cT2, a1, a2, f2, B, bsB, cB2, out, bsO, tmp1);
@@ -1056,7 +1056,7 @@ struct pepsvmc_ctx {
       return fused4(fused4_right(E, bsE, cT2, cB2, T, bsT, cT, a1, f1, a2, f2, B, bsB, cB, out, bsO));
     const Env4Fused f = fused4_right(E, bsE, cT2, cB2, T, bsT, cT, a1, f1, a2, f2, B, bsB, cB, out, bsO);
     const Env4Outs o{{out}};
-    if (f32_fused() && env4_f32_fits(f, o)) return step4_f32(f, o, true);
+    if (f32_fused() && env4_f32_takes(f, o, C)) return step4_f32(f, o, true);
     const int D1l = a1.Dl, D1r = a1.Dr, Du1 = a1.Du, Dd1 = a1.Dd;
     const int D2l = a2.Dl, D2r = a2.Dr, Dd2 = a2.Dd;
     GemmDesc g;
@@ -1557,7 +1557,7 @@ struct pepsvmc_ctx {
       const Env4Fused f4 = fused4_left(Lin, bsL, tb[m], bb[m], T.site(m), T.chain_stride, tb[m + 1], a1[m], 0, a2[m], 0,
                                        B.site(m), B.chain_stride, bb[m + 1], cur, S4);
       const Env4Outs o4{{cur, Pbn, Ptn, fl4}};
-      const bool f32 = f32_fused() && env4_f32_fits(f4, o4);
+      const bool f32 = f32_fused() && env4_f32_takes(f4, o4, C);
       if (fz) {
         PV_CUDA(step(Lin, bsL, 0, 0, cur));
       } else if (f32) {
@@ -2195,7 +2195,7 @@ int pepsvmc_env4_left(pepsvmc_ctx* x, const float* E, const float* T, const floa
   if (bmajor) return x->fail(PEPSVMC_EINVAL, "env4_left: the b-major layout needs the fused kernel");
   const Env4Outs outs{{out}};
   const long long no = n_chains * f.bsO;
-  if (x->f32_fused() && env4_f32_fits(f, outs) && !overlaps(out, no, E, n_chains * f.bsE) &&
+  if (x->f32_fused() && env4_f32_takes(f, outs, n_chains) && !overlaps(out, no, E, n_chains * f.bsE) &&
       !overlaps(out, no, T, n_chains * f.bsT) && !overlaps(out, no, A1, 2 * s1) && !overlaps(out, no, A2, 2 * s2) &&
       !overlaps(out, no, B, n_chains * f.bsB) && !overlaps(out, no, spins1, n_chains) &&
       !overlaps(out, no, spins2, n_chains)) {

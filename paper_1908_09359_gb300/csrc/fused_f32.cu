@@ -365,9 +365,21 @@ __global__ void __maxnreg__(80) env4_f32_kernel(const Env4Fused a, const Env4Out
   }
 }
 
-// Threads of a CTA: enough for the first products' tasks of 8 x 4, at most 256, or 512 where the
-// shared memory lets an SM hold one CTA only.
-int threads_for(int tasks, int smem) {
+// Threads of a CTA.  Where CTAs share an SM: enough for the first products' tasks of 8 x 4, at most 256,
+// or 512 where the shared memory lets an SM hold one CTA only.  A CTA that has an SM to itself is
+// bound by the latency of its products, and takes as many threads as have work in the narrow tiles
+// (run: 4 x 2, four times the tasks).  Measured over 580 steps of up to 152 CTAs, these / as where
+// CTAs share: 0.89-0.96 of the time up to 16 tasks, 0.67-0.73 from 17 to 64, 0.82-0.86 to 128, 0.92-0.95
+// above 256 (128 tasks fill 128 threads at once: 384 take 1.18 of the time); over 66 of up to 304 CTAs
+// 0.72-0.84 from 17 to 64 tasks.  With 64 threads, few
+// chains were slower than in separate products (Dc 18, D 5, 4 chains 14.8 us against 11.0; now 7.5).
+int threads_for(int tasks, int smem, long long blocks, int sms) {
+  if (blocks <= sms) {
+    if (tasks < 128) return tasks > 64 ? 384 : tasks > 4 ? 256 : 64;
+    if (tasks == 128) return 128;
+    return tasks > 256 ? 512 : 256;
+  }
+  if (blocks <= 2LL * sms && tasks > 16 && tasks <= 64) return 256;
   return tasks > 256 && 2 * (smem + 1024) > 228 * 1024 ? 512 : tasks > 128 ? 256 : tasks > 64 ? 128 : 64;
 }
 
@@ -391,9 +403,11 @@ cudaError_t env3_f32(const Env3Fused& a, float* out1, bool rev2, bool rev3, cons
   const long long blocks = (long long)a.batch * ((a.cT2 + kTA - 1) / kTA);
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int tasks = a.Du * ((a.Dl * a.cB + 3) / 4), tasks2 = a.cB * ((a.Dr * a.Dd + 3) / 4);
+  int sms = 0;
+  PV_CUDA(sm_count(&sms));
   auto* kernel = mid.p ? env3_f32_kernel<true> : env3_f32_kernel<false>;
   if (smem > 48 * 1024) PV_CUDA(allow_smem(kernel, kMaxSmem));
-  return launch_early(kernel, (unsigned)blocks, threads_for(tasks > tasks2 ? tasks : tasks2, smem), smem, st, a, out1, rev2, rev3, mid);
+  return launch_early(kernel, (unsigned)blocks, threads_for(tasks > tasks2 ? tasks : tasks2, smem, blocks, sms), smem, st, a, out1, rev2, rev3, mid);
 }
 
 static bool several(const Env4Outs& o) { return (o.p[0] != nullptr) + (o.p[1] != nullptr) + (o.p[2] != nullptr) + (o.p[3] != nullptr) > 1; }
@@ -404,6 +418,20 @@ bool env4_f32_fits(const Env4Fused& a, const Env4Outs& outs) {
          tile_in_32_bits(a.cT, a.sTa, a.Du1, a.sTu, a.sTa2);
 }
 
+// Up to 8 CTAs the chip is empty either way: the step takes the time of one CTA, about 80,000
+// multiply-adds per us, the separate products 5.5 us each (they spread a chain over many CTAs).
+// Measured, separate / this: one chain of Dc 15, D 6 23.9 / 33.0 us, 2 chains of Dc 12, D 6 22.3 / 26.1, 4
+// of Dc 15, D 5 21.1 / 22.3, one of Dc 16, D 4 20.3 / 9.9.
+bool env4_f32_takes(const Env4Fused& a, const Env4Outs& outs, int chains) {
+  if (!env4_f32_fits(a, outs)) return false;
+  if ((long long)chains * ((a.cT2 + kTA - 1) / kTA) > 8) return true;
+  const int n0 = (outs.p[0] != nullptr) + (outs.p[1] != nullptr), n1 = (outs.p[2] != nullptr) + (outs.p[3] != nullptr);
+  const int flips = (n0 > 0) + (n1 > 0), n = n0 + n1;
+  const double s1 = (double)a.D1l * a.D2l * a.cB * a.Du1 * a.cT, s2 = (double)a.D2l * a.cB * a.D1r * a.Dd1 * a.D1l * a.Du1,
+               s3 = (double)a.cB * a.D1r * a.D2r * a.Dd2 * a.D2l * a.Dd1, s4 = (double)a.D1r * a.D2r * a.cB2 * a.cB * a.Dd2;
+  return kTA * (s1 + flips * s2 + n * (s3 + s4)) <= 5.5 * 80e3 * (1 + flips + 2 * n);
+}
+
 cudaError_t env4_f32(const Env4Fused& a, const Env4Outs& outs, bool rev, cudaStream_t st) {
   if (g_dry_run || a.batch <= 0) return cudaSuccess;
   int off[7];
@@ -412,7 +440,9 @@ cudaError_t env4_f32(const Env4Fused& a, const Env4Outs& outs, bool rev, cudaStr
   const long long blocks = (long long)a.batch * ((a.cT2 + kTA - 1) / kTA);
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int tasks = a.D2l * a.cB * ((a.D1r * a.Dd1 + 3) / 4);
-  return launch_early(env4_f32_kernel, (unsigned)blocks, threads_for(tasks, smem), smem, st, a, outs, several(outs), rev);
+  int sms = 0;
+  PV_CUDA(sm_count(&sms));
+  return launch_early(env4_f32_kernel, (unsigned)blocks, threads_for(tasks, smem, blocks, sms), smem, st, a, outs, several(outs), rev);
 }
 
 }  // namespace pv

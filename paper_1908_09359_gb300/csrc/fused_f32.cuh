@@ -24,6 +24,8 @@ struct Env4Outs {
   float* p[4] = {};
 };
 bool env4_f32_fits(const Env4Fused& a, const Env4Outs& outs);
+// Whether it fits and is faster than the separate products at this number of chains.
+bool env4_f32_takes(const Env4Fused& a, const Env4Outs& outs, int chains);
 cudaError_t env4_f32(const Env4Fused& a, const Env4Outs& outs, bool rev, cudaStream_t st);
 
 }  // namespace pv

@@ -164,6 +164,7 @@ int fake_launches() { return (int)launches.size(); }
 void fake_clear() { launches.clear(); }
 const char* fake_name(int i) { return launches[i].name.c_str(); }
 long long fake_grid(int i) { return (long long)launches[i].grid.x * launches[i].grid.y * launches[i].grid.z; }
+int fake_threads(int i) { return (int)(launches[i].block.x * launches[i].block.y * launches[i].block.z); }
 long long fake_smem(int i) { return (long long)launches[i].smem; }
 
 // ---- the library's launchers by plain arguments; d: bonds and legs in the order of the C ABI
@@ -174,7 +175,7 @@ int host_env3_f32_fits(int n, const int* d) {
   f.sTa = (long long)f.Du * f.cT2; f.sTu = f.cT2; f.sTa2 = 1;
   return pv::env3_f32_fits(f);
 }
-int host_env4_f32_fits(int n, const int* d, int variants) {
+static int env4_f32_question(int n, const int* d, int variants, bool takes) {
   pv::Env4Fused f;
   f.batch = n;
   f.cT = d[0]; f.cB = d[1]; f.cT2 = d[2]; f.cB2 = d[3];
@@ -183,8 +184,10 @@ int host_env4_f32_fits(int n, const int* d, int variants) {
   f.sTa = (long long)f.Du1 * f.cT2; f.sTu = f.cT2; f.sTa2 = 1;
   pv::Env4Outs o;
   for (int i = 0; i < variants; ++i) o.p[i] = (float*)16;
-  return pv::env4_f32_fits(f, o);
+  return takes ? pv::env4_f32_takes(f, o, n) : pv::env4_f32_fits(f, o);
 }
+int host_env4_f32_fits(int n, const int* d, int variants) { return env4_f32_question(n, d, variants, false); }
+int host_env4_f32_takes(int n, const int* d, int variants) { return env4_f32_question(n, d, variants, true); }
 
 static float* at(int k) { return (float*)((uintptr_t)k << 44); }  // far apart and aligned
 static pv::Env3Fused env3(int n, int chi, int D) {
@@ -252,6 +255,7 @@ int host_normalize(int n, int arrays, int chains) {
   return pv::k_normalize_pow2(at(1), n, n, arrays > 1 ? at(2) : nullptr, n, arrays > 1 ? n : 0, arrays > 2 ? at(3) : nullptr, n,
                               arrays > 2 ? n : 0, (int*)at(4), chains, &status, nullptr);
 }
+int host_env3_f32(int n, int chi, int D) { return pv::env3_f32(env3(n, chi, D), nullptr, false, false, pv::Mid3(), nullptr); }
 int host_gemm_tc(int mode, int bn) {
   pv::GemmDesc g;
   g.M = g.N = g.K = 128;

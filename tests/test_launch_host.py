@@ -206,3 +206,23 @@ def test_three_line_step_takes_the_faster_form(fake, n, chi, D, mode, kernel):
 @pytest.mark.parametrize("n,cV,kernel", [(152, 12, "fused"), (192, 12, "tile"), (304, 16, "tile"), (305, 16, "fused"), (192, 17, "fused")])
 def test_optimal_site_takes_the_faster_form(fake, n, cV, kernel):
     assert fake.host_proj3(n, 24, cV, 6, 3) == OK and f"proj3_{kernel}_kernel" in fake.fake_name(0).decode()
+
+
+@pytest.mark.parametrize("n,chi,D,threads", [
+    (4, 27, 2, 256), (64, 16, 4, 256), (76, 16, 4, 256), (77, 16, 4, 256), (152, 16, 4, 256), (153, 16, 4, 64), (1, 2, 1, 64),
+    (4, 18, 5, 384), (153, 18, 5, 128), (4, 16, 5, 384), (2, 30, 8, 512), (2048, 24, 6, 256),
+])
+def test_threads_of_fp32_steps(fake, n, chi, D, threads):
+    """A CTA with an SM to itself takes enough threads for narrow tiles (64 threads made few chains slower
+    than the separate products)."""
+    # the context-free entry point's fixed scratch bounds its sizes; the launcher itself does not
+    assert fake.host_env3_f32(n, chi, D) == OK and fake.fake_threads(0) == threads
+
+
+@pytest.mark.parametrize("n,chi,D,variants,takes", [(1, 15, 6, 1, 0), (4, 12, 6, 1, 0), (5, 12, 6, 1, 1), (1, 15, 6, 4, 0), (1, 16, 4, 1, 1),
+                                                    (1, 16, 4, 4, 1), (4, 15, 5, 1, 1), (1, 4, 2, 4, 1)])
+def test_few_chains_of_large_four_line_steps_take_the_separate_products(fake, n, chi, D, variants, takes):
+    d = (C.c_int * 11)(chi, chi, chi, chi, *[D] * 7)
+    assert fake.host_env4_f32_takes(n, d, variants) == takes
+    if variants == 1:
+        assert fake.host_env4_f32_fits(n, d, variants) == 1
