@@ -29,6 +29,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -44,9 +45,9 @@ UNIT = "samples/s"
 FP32_ALU_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 
 # DRAM traffic of one bulk launch of each fused step (Dc 32, D 8), dram__bytes_read.sum +
-# dram__bytes_write.sum from one ncu capture of the kernel whose source hashed to
-# `source_sha`, per chain of that capture; the bench reports it only while the source is
-# unchanged.
+# dram__bytes_write.sum from one ncu capture of the kernel whose source (with the headers it
+# includes) hashed to `source_sha`, per chain of that capture; the bench reports it only while
+# the source is unchanged.
 NCU_TRAFFIC = {
     "fused4": {"bytes_per_chain": (206.169600e6 + 98.996224e6) / 512,
                "source": "paper_1908_09359_gb300/csrc/fused_env4_pipe.cu", "source_sha": "da40db441c68df59",
@@ -239,8 +240,32 @@ def kernel_groups(shapes):
 
 
 def source_sha(rel):
-    with open(os.path.join(ROOT, rel), "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+    """Hash of a source file and of every header it includes from its own folder, theirs included
+    (a kernel's loads and stores lie in both)."""
+    files, todo = {}, [rel]
+    while todo:
+        r = todo.pop()
+        if r in files:
+            continue
+        with open(os.path.join(ROOT, r), "rb") as f:
+            files[r] = f.read()
+        for name in re.findall(rb'^\s*#\s*include\s+"([^"]+)"', files[r], re.M):
+            inc = os.path.join(os.path.dirname(r), name.decode())
+            if os.path.exists(os.path.join(ROOT, inc)):
+                todo.append(inc)
+    h = hashlib.sha256()
+    for r in sorted(files):
+        h.update(r.encode() + b"\0" + files[r] + b"\0")
+    return h.hexdigest()[:16]
+
+
+def fused_kernel(group, bulk):
+    """The kernel behind a group of fused steps: the bulk shape's (full bonds), else those the
+    group's shapes are shared between."""
+    if group == "fused4":
+        return "env4_pipe_kernel" if bulk else "env4_pipe_kernel and env4_fused_kernel"
+    name = {"fused3": "env3", "fusedP": "proj3"}[group]
+    return f"{name}_fused_kernel" if bulk else f"{name}_fused_kernel and {name}_tile_kernel"
 
 
 # ------------------------------------------------------------------ the oracle on the host
@@ -586,10 +611,12 @@ def run_ours(args):
             traffic = t["bytes_per_chain"] * C
         step_flops = prof["gemm_flops"]
         roofline = {
-            "kernel": {"fused4": "env4_pipe_kernel (four-line column step, tcgen05, split BF16)",
-                       "fused3": "env3_fused_kernel (three-line column step, tcgen05, split BF16)",
-                       "fusedP": "proj3_fused_kernel (optimal site of the truncation fit, tcgen05, split BF16)",
-                       "f32_fused": "env3_f32_kernel, env4_f32_kernel (column steps and optimal sites, FP32 CUDA cores)",
+            "kernel": fused_kernel(dominant, rec is bulk) +
+                      {"fused4": " (four-line column step, tcgen05, split BF16)",
+                       "fused3": " (three-line column step, tcgen05, split BF16)",
+                       "fusedP": " (optimal site of the truncation fit, tcgen05, split BF16)"}[dominant]
+                      if dominant.startswith("fused") else
+                      {"f32_fused": "env3_f32_kernel, env4_f32_kernel (column steps and optimal sites, FP32 CUDA cores)",
                        "gemm_tc": "gemm_tc_kernel (separate products, tcgen05)",
                        "gemm_f32": "gemm_f32_kernel (separate products, FP32 CUDA cores)"}[dominant],
             "shape": rec["shape"], "bound": primary["bound"], "achieved": primary["achieved"],
