@@ -427,10 +427,12 @@ cudaError_t qr_pos_batched(const float* Y, long long bsY, long long yrs, long lo
   if (cols > kQrMaxCols || rows < cols || cols <= 0) return cudaErrorInvalidValue;
   if (rows <= 256 && cols <= kQrRegCols) {
     // the fewest warps that cover the rows with RPT = 2; RPT = 4 once an SM holds more than two
-    // matrices of the full width (304 matrices on 152 SMs; figures above)
+    // matrices of the full width (figures above)
     if (rows <= 64) return launch_tree<2, 1>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols, batch, st);
     if (rows <= 128) return launch_tree<2, 2>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols, batch, st);
-    if (cols > 24 && batch > 304)
+    int sms = 0;
+    PV_CUDA(sm_count(&sms));
+    if (cols > 24 && batch > 2 * sms)
       return launch_early(qr_pos_tree_kernel<4, 2, 4>, batch, 64, 0, st, Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols);
     return launch_tree<2, 4>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols, batch, st);
   }

@@ -226,3 +226,10 @@ def test_few_chains_of_large_four_line_steps_take_the_separate_products(fake, n,
     assert fake.host_env4_f32_takes(n, d, variants) == takes
     if variants == 1:
         assert fake.host_env4_f32_fits(n, d, variants) == 1
+
+
+@pytest.mark.parametrize("device,batch,rows_per_thread", [(0, 304, 2), (0, 305, 4), (1, 152, 2), (1, 153, 4)])
+def test_qr_form_follows_the_matrices_per_sm(fake, device, batch, rows_per_thread):
+    fake.fake_device(device)
+    assert fake.pepsvmc_qr_pos(E, OUT, batch, 256, 32, 0, None) == OK
+    assert f"qr_pos_tree_kernelILi{rows_per_thread}E" in fake.fake_name(0).decode()
