@@ -372,7 +372,8 @@ __global__ void __maxnreg__(80) env4_f32_kernel(const Env4Fused a, const Env4Out
 // CTAs share: 0.89-0.96 of the time up to 16 tasks, 0.67-0.73 from 17 to 64, 0.82-0.86 to 128, 0.92-0.95
 // above 256 (128 tasks fill 128 threads at once: 384 take 1.18 of the time); over 66 of up to 304 CTAs
 // 0.72-0.84 from 17 to 64 tasks.  With 64 threads, few
-// chains were slower than in separate products (Dc 18, D 5, 4 chains 14.8 us against 11.0; now 7.5).
+// chains were slower than in separate products (a ragged step of Dc 19, 4 chains 14.8 us against
+// 11.0; now 7.5).
 int threads_for(int tasks, int smem, long long blocks, int sms) {
   if (blocks <= sms) {
     if (tasks < 128) return tasks > 64 ? 384 : tasks > 4 ? 256 : 64;
@@ -418,18 +419,31 @@ bool env4_f32_fits(const Env4Fused& a, const Env4Outs& outs) {
          tile_in_32_bits(a.cT, a.sTa, a.Du1, a.sTu, a.sTa2);
 }
 
-// Up to 8 CTAs the chip is empty either way: the step takes the time of one CTA, about 80,000
-// multiply-adds per us, the separate products 5.5 us each (they spread a chain over many CTAs).
-// Measured, separate / this: one chain of Dc 15, D 6 23.9 / 33.0 us, 2 chains of Dc 12, D 6 22.3 / 26.1, 4
-// of Dc 15, D 5 21.1 / 22.3, one of Dc 16, D 4 20.3 / 9.9.
+// Passes over k of one product, in passes of the wide tile (run).
+static double passes(double ni, double nc, double K, int threads) {
+  const double wide = ni * ceil(nc / 4);
+  return 2 * wide > threads ? ceil(wide / threads) * K : 0.5 * ceil(ni * 2 * ceil(nc / 2) / threads) * K;
+}
+
+// A CTA alone on its SM takes about 0.14 us per pass, however few others there are; the separate
+// products spread a chain over many CTAs: 5.5 us a launch, and 3.9e6 multiply-adds per us once the
+// chip is full.  Measured, separate / this: one chain of Dc 15, D 6 23.9 / 33.0 us, 3 of Dc 17, D 5 22.9 /
+// 28.0, 2 of Dc 12, D 6 22.3 / 26.1, one of Dc 16, D 4 20.3 / 9.9.
 bool env4_f32_takes(const Env4Fused& a, const Env4Outs& outs, int chains) {
   if (!env4_f32_fits(a, outs)) return false;
-  if ((long long)chains * ((a.cT2 + kTA - 1) / kTA) > 8) return true;
+  const long long blocks = (long long)chains * ((a.cT2 + kTA - 1) / kTA);
+  int sms = 0, off[7];
+  if (sm_count(&sms) != cudaSuccess || blocks > sms) return true;
   const int n0 = (outs.p[0] != nullptr) + (outs.p[1] != nullptr), n1 = (outs.p[2] != nullptr) + (outs.p[3] != nullptr);
   const int flips = (n0 > 0) + (n1 > 0), n = n0 + n1;
-  const double s1 = (double)a.D1l * a.D2l * a.cB * a.Du1 * a.cT, s2 = (double)a.D2l * a.cB * a.D1r * a.Dd1 * a.D1l * a.Du1,
-               s3 = (double)a.cB * a.D1r * a.D2r * a.Dd2 * a.D2l * a.Dd1, s4 = (double)a.D1r * a.D2r * a.cB2 * a.cB * a.Dd2;
-  return kTA * (s1 + flips * s2 + n * (s3 + s4)) <= 5.5 * 80e3 * (1 + flips + 2 * n);
+  const int t = threads_for(a.D2l * a.cB * ((a.D1r * a.Dd1 + 3) / 4), layout4(a, several(outs), off) * 4, blocks, sms);
+  const double E = (double)a.D1l * a.D2l * a.cB, Y = (double)a.D2l * a.cB, r1d1 = (double)a.D1r * a.Dd1, l1u1 = (double)a.D1l * a.Du1,
+               Z = (double)a.cB * a.D1r, r2d2 = (double)a.D2r * a.Dd2, l2d1 = (double)a.D2l * a.Dd1, O = (double)a.D1r * a.D2r,
+               bd2 = (double)a.cB * a.Dd2;
+  const double here = 0.14 * (passes(a.Du1, E, a.cT, t) + flips * passes(Y, r1d1, l1u1, t) +
+                              n * (passes(Z, r2d2, l2d1, t) + passes(O, a.cB2, bd2, t)));
+  const double adds = chains * (double)a.cT2 * (a.Du1 * E * a.cT + flips * Y * r1d1 * l1u1 + n * (Z * r2d2 * l2d1 + O * a.cB2 * bd2));
+  return here <= 5.5 * (1 + flips + 2 * n) + adds / 3.9e6;
 }
 
 cudaError_t env4_f32(const Env4Fused& a, const Env4Outs& outs, bool rev, cudaStream_t st) {

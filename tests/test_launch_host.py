@@ -219,8 +219,8 @@ def test_threads_of_fp32_steps(fake, n, chi, D, threads):
     assert fake.host_env3_f32(n, chi, D) == OK and fake.fake_threads(0) == threads
 
 
-@pytest.mark.parametrize("n,chi,D,variants,takes", [(1, 15, 6, 1, 0), (4, 12, 6, 1, 0), (5, 12, 6, 1, 1), (1, 15, 6, 4, 0), (1, 16, 4, 1, 1),
-                                                    (1, 16, 4, 4, 1), (4, 15, 5, 1, 1), (1, 4, 2, 4, 1)])
+@pytest.mark.parametrize("n,chi,D,variants,takes", [(1, 15, 6, 1, 0), (1, 12, 6, 1, 0), (30, 12, 6, 1, 1), (3, 17, 5, 1, 0), (100, 17, 5, 1, 1),
+                                                    (1, 15, 6, 4, 0), (1, 16, 4, 1, 1), (1, 16, 4, 4, 1), (1, 4, 2, 4, 1)])
 def test_few_chains_of_large_four_line_steps_take_the_separate_products(fake, n, chi, D, variants, takes):
     d = (C.c_int * 11)(chi, chi, chi, chi, *[D] * 7)
     assert fake.host_env4_f32_takes(n, d, variants) == takes
