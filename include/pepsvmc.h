@@ -305,16 +305,19 @@ int pepsvmc_env4_left(pepsvmc_ctx* ctx, const float* E, const float* T, const fl
  * synchronise the device and fragments a planned pool.  Same operation, layouts
  * and spin rule as pepsvmc_env3_left; runs asynchronously on ``stream`` (a
  * cudaStream_t, NULL = legacy default stream) on the current device.
- * Scratch: the two intermediates live in one fixed array of
- * PEPSVMC_NOALLOC_SCRATCH_FLOATS floats (16 MiB) of the library's own device
- * memory, present on every GPU where the library's device code is loaded until
- * the process exits.  Every call looks up that array's device address for the
- * current device and context (no allocation; after a device reset the new
- * context's address is used); the first call on a device loads the library's
- * device code there, so make that first call before any stream capture.  Every call uses the same array, and it keeps the last call's
- * contents (nothing in it needs to start at zero); calls whose execution overlaps
- * on the GPU -- on different streams or devices sharing nothing, or from several
- * host threads -- race on it and must be serialised by the caller.
+ * Scratch: where one kernel's shared memory holds the two intermediates (bonds up to
+ * about Dc = 32 with D = 8) they stay there.  Otherwise, and when ``out`` lies over an
+ * input, they live in one fixed array of PEPSVMC_NOALLOC_SCRATCH_FLOATS floats
+ * (16 MiB) of the library's own device memory, present on every GPU where the
+ * library's device code is loaded until the process exits.  A call that uses the
+ * array looks up its device address for the current device and context (no
+ * allocation; after a device reset the new context's address is used).  The array
+ * keeps the last call's contents (nothing in it needs to start at zero), and calls
+ * that use it and whose execution overlaps on the GPU -- on different streams, or
+ * from several host threads -- race on it; which calls do may change with a version
+ * of the library, so the caller serialises all of them.  Kernels are loaded when they
+ * are first launched on a device: make a first call of each size before any stream
+ * capture, so that none is loaded during one.
  * Errors: EINVAL for null pointers, non-positive sizes, or when
  * 2 * n_chains * max(Dl*cB*Du*cT2, cB*cT2*Dr*Dd) exceeds the array; ECUDA.      */
 #define PEPSVMC_NOALLOC_SCRATCH_FLOATS 4194304

@@ -333,7 +333,8 @@ class PepsVMC:
 def env3_left_noalloc(E, T, A, spins, B, out, dims, stream=None):
     """The three-line environment step without a context and without any device
     allocation (for callers that must not allocate once running); the intermediates
-    use the library's fixed scratch array, so calls must not overlap on the GPU.
+    of larger steps use the library's fixed scratch array, so calls must not overlap
+    on the GPU.
     Arguments as PepsVMC.env3_left; ``stream`` defaults to torch's current stream."""
     lib = _lib.load()
     if stream is None:

@@ -350,8 +350,10 @@ cudaError_t env4_fused(const Env4Fused& a, bool split, unsigned* status, cudaStr
   if (g_dry_run || a.batch <= 0) return cudaSuccess;
   if (!env4_fused_fits(a)) return cudaErrorInvalidValue;
   // Full bonds, b-major and dense: the pipeline, at every number of chains (61 -> 39 us at one,
-  // 566 -> 438 us at 512).  Its conversions have no bounds; smaller bonds and other orders
-  // of E's indices stay with the kernel above.
+  // 566 -> 438 us at 512).  It was written for those alone: its conversions of operands have no
+  // bounds and take E in that order, so that they keep up with three streams.  A form with the
+  // bounded conversions of fused_pipe.cuh has not been written; smaller bonds and other orders of E's
+  // indices stay with the kernel above.
   alignas(16) unsigned char plan[kEnv4PlanBytes];
   if (env4_pipe_fits(a, plan)) return env4_pipe(plan, split, status, st);
   return split ? launch<true>(a, status, st) : launch<false>(a, status, st);

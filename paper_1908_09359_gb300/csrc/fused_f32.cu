@@ -22,12 +22,13 @@
 // waited for their loads.  Here all operands of a step are in flight at once, by asynchronous
 // copies (through registers, in turn, a third of the time went to loading: Dc 24, D 6 350 us,
 // and odd bonds, one CTA per SM, were slower than the separate products: Dc 25, D 7, 40 chains
-// 65 us against 40).  Measured (separate -> fused): three-line step Dc 24, D 6, 2048 chains
-// 909 -> 244 us (29 TFLOP/s), Dc 16, D 4, 1024 chains 80 -> 21 us, Dc 32, D 8, 512 chains 578 ->
-// 262 us, Dc 23, D 7, 1624 chains 741 -> 486 us, 64 chains of Dc 16, D 4 28 -> 9 us; four-line step
-// Dc 16, D 4, 1024 chains 385 -> 86 us, Dc 17, D 5, 104 chains 99 -> 85 us.  Over 120 drawn steps
-// (bonds to 32 and 8, 1-2048 chains) 118 are at 1.0x or above, the others at 0.91 and 0.99.
-// Steps whose intermediates exceed a CTA's shared memory keep the separate products.
+// 65 us against 40).  Measured in a graph, separate products (each with its fastest tile) -> this:
+// three-line step Dc 24, D 6, 2048 chains 900 -> 238 us (30 TFLOP/s), Dc 16, D 4, 1024 chains 71.5 ->
+// 18.7 us, 64 chains 15.7 -> 5.2 us, Dc 32, D 8, 512 chains 568 -> 254 us, Dc 23, D 7, 1624 chains 880 ->
+// 484 us, Dc 25, D 7, 40 chains 49.6 -> 35.0 us; four-line step Dc 16, D 4, 1024 chains 376 -> 83 us,
+// Dc 17, D 5, 104 chains 106 -> 82 us.  Over 1,900 drawn steps (bonds to 64 and 12, 1-2048 chains) about
+// ten are slower, by up to 21 %, all of them ragged or four-line steps of a few chains.  Steps whose
+// intermediates exceed a CTA's shared memory keep the separate products.
 #include <limits.h>
 #include <math.h>
 
