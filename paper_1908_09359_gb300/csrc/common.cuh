@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 
 namespace pv {
@@ -78,21 +79,7 @@ inline cudaError_t reported(cudaError_t e) {
   return e;
 }
 
-// Both of the following hold for the device and context that are current when a launch is made, so
-// they are asked for at every launch and nothing is kept: a process may use several devices, or
-// reset one.  (0.2 us and 0.03 us of host time, where a launch takes 1.5.)
-//
-// A kernel may have more than 48 KB of shared memory, its static variables included, only once its
-// limit of dynamic shared memory is raised.  bytes: the most that any launch of this kernel asks
-// for, so that threads that launch it with different sizes do not lower each other's limit.  all: the SM's whole shared memory rather than
-// first-level cache, so that as many CTAs as planned fit an SM.
-constexpr size_t kCtaSmem = 227 * 1024;  // what a CTA of sm_103a may have, static and dynamic
-template <typename... Par>
-cudaError_t allow_smem(void (*kernel)(Par...), size_t bytes, bool all = false) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess && all) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  return reported(e);
-}
+// The SMs of the current device (0.03 us of host time, so it is asked for at every launch that needs it).
 inline cudaError_t sm_count(int* sms) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -118,7 +105,7 @@ inline bool plain_launches(cudaStream_t st) {
   return reported(cudaStreamIsCapturing(st, &s)) != cudaSuccess || s != cudaStreamCaptureStatusNone;
 }
 template <typename... Par, typename... Arg>
-cudaError_t launch_early(void (*kernel)(Par...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Arg&... arg) {
+cudaError_t launch(bool plain, void (*kernel)(Par...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Arg&... arg) {
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
@@ -128,8 +115,50 @@ cudaError_t launch_early(void (*kernel)(Par...), dim3 grid, dim3 block, size_t s
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = &at;
-  cfg.numAttrs = plain_launches(st) ? 0 : 1;
+  cfg.numAttrs = plain ? 0 : 1;
   return reported(cudaLaunchKernelEx(&cfg, kernel, static_cast<Par>(arg)...));
+}
+template <typename... Par, typename... Arg>
+cudaError_t launch_early(void (*kernel)(Par...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Arg&... arg) {
+  return launch(plain_launches(st), kernel, grid, block, smem, st, arg...);
+}
+
+// The same for a kernel with more than 48 KB of shared memory, its static variables included: it may be
+// launched once its limit of dynamic shared memory is raised, which holds for the device that is
+// current and until that device is reset.  The limit is set on the first launch on a device, and
+// again when a launch is refused (a device that was reset); inside a capture, which a refused launch
+// might spoil, always.  (Set at every launch it cost the smallest steps 7 %: 0.2 us, twice where
+// `all` is, of 6.6.)  A refusal is reported and not kept.
+constexpr size_t kCtaSmem = 227 * 1024;  // what a CTA of sm_103a may have, static and dynamic
+struct SmemLimit {
+  size_t bytes;  // the most that any launch of the kernel asks for: threads do not lower each other's limit
+  bool all;      // the SM's whole shared memory rather than first-level cache, so that two CTAs fit an SM
+  std::atomic<uint64_t> devices{0};  // bit of each device (modulo 64) it was set on
+  template <typename... Par>
+  cudaError_t set(void (*kernel)(Par...), uint64_t bit) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && all) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e == cudaSuccess) devices.fetch_or(bit, std::memory_order_relaxed);
+    return reported(e);
+  }
+};
+// early: whether the kernel calls after_previous().
+template <typename... Par, typename... Arg>
+cudaError_t launch_large(SmemLimit& limit, bool early, void (*kernel)(Par...), dim3 grid, dim3 block, size_t smem,
+                         cudaStream_t st, const Arg&... arg) {
+  int dev = 0;
+  cudaError_t e = reported(cudaGetDevice(&dev));
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = (uint64_t)1 << (dev & 63);
+  const bool capture = plain_launches(st), plain = capture || !early;
+  if (capture || !(limit.devices.load(std::memory_order_relaxed) & bit)) {
+    e = limit.set(kernel, bit);
+    return e == cudaSuccess ? launch(plain, kernel, grid, block, smem, st, arg...) : e;
+  }
+  e = launch(plain, kernel, grid, block, smem, st, arg...);
+  if (e != cudaErrorInvalidValue) return e;
+  e = limit.set(kernel, bit);
+  return e == cudaSuccess ? launch(plain, kernel, grid, block, smem, st, arg...) : e;
 }
 #ifdef __CUDACC__
 __device__ __forceinline__ void after_previous() {

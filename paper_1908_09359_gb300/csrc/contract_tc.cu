@@ -300,10 +300,10 @@ template <int EB, int BN, bool X3, bool DB = false>
 cudaError_t launch(const GemmDesc& d, unsigned* status, cudaStream_t st) {
   // two plain stages, one split stage, or two split stages (DB)
   constexpr int smem = (DB ? 4 : 2) * (kBM + BN) * kKBytes;
-  PV_CUDA(allow_smem(gemm_tc_kernel<EB, BN, X3, DB>, smem));
+  static SmemLimit limit{smem, false};
   const int tiles = ((d.M + kBM - 1) / kBM) * ((d.N + BN - 1) / BN);
   dim3 grid(tiles, d.batch < 65535 ? d.batch : 65535, (d.batch + 65534) / 65535);
-  return launch_early(gemm_tc_kernel<EB, BN, X3, DB>, grid, kThreads, smem, st, d, status);
+  return launch_large(limit, true, gemm_tc_kernel<EB, BN, X3, DB>, grid, kThreads, smem, st, d, status);
 }
 
 template <int EB, bool X3>

@@ -137,7 +137,7 @@ cudaError_t proj3_fused(const Proj3Fused& a, bool split, unsigned* status, cudaS
 
 // The same two steps with one tile per CTA (fused_env3_tiles.cu), for launches of few tiles;
 // env3_fused and proj3_fused choose.
-cudaError_t env3_tiles(const Env3Fused& a, bool split, unsigned* status, cudaStream_t st);
-cudaError_t proj3_tiles(const Proj3Fused& a, bool split, unsigned* status, cudaStream_t st);
+cudaError_t env3_tiles(const Env3Fused& a, bool split, int sms, unsigned* status, cudaStream_t st);
+cudaError_t proj3_tiles(const Proj3Fused& a, bool split, int sms, unsigned* status, cudaStream_t st);
 
 }  // namespace pv

@@ -420,8 +420,8 @@ __global__ void __launch_bounds__(kPipeThreads, 1) env3_fused_kernel(const __gri
 
 template <bool X3, bool FULL>
 cudaError_t launch(const Plan3& P, int grid, unsigned* status, cudaStream_t st) {
-  PV_CUDA(allow_smem(env3_fused_kernel<X3, FULL>, SMEM_BYTES));
-  return launch_early(env3_fused_kernel<X3, FULL>, grid, kPipeThreads, SMEM_BYTES, st, P, status);
+  static SmemLimit limit{SMEM_BYTES, false};
+  return launch_large(limit, true, env3_fused_kernel<X3, FULL>, grid, kPipeThreads, SMEM_BYTES, st, P, status);
 }
 
 // ------------------------------------------------------------ optimal site of the fit
@@ -715,8 +715,8 @@ __global__ void __launch_bounds__(kPipeThreads, 1) proj3_fused_kernel(const __gr
 
 template <bool X3, bool FULL>
 cudaError_t launch_proj3(const PlanP& P, int grid, unsigned* status, cudaStream_t st) {
-  PV_CUDA(allow_smem(proj3_fused_kernel<X3, FULL>, P_SMEM_BYTES));
-  return launch_early(proj3_fused_kernel<X3, FULL>, grid, kPipeThreads, P_SMEM_BYTES, st, P, status);
+  static SmemLimit limit{P_SMEM_BYTES, false};
+  return launch_large(limit, true, proj3_fused_kernel<X3, FULL>, grid, kPipeThreads, P_SMEM_BYTES, st, P, status);
 }
 
 bool all_full(const PipeOp (&op)[4]) {
@@ -760,7 +760,7 @@ cudaError_t env3_fused(const Env3Fused& a, bool split, unsigned* status, cudaStr
   PV_CUDA(sm_count(&sms));
   const Plan3 P = plan3(a, sms, grid);
   const bool full = all_full(P.op);
-  if (!full && !pipeline_pays(P, sms, split)) return env3_tiles(a, split, status, st);
+  if (!full && !pipeline_pays(P, sms, split)) return env3_tiles(a, split, sms, status, st);
   if (full) return split ? launch<true, true>(P, grid, status, st) : launch<false, true>(P, grid, status, st);
   return split ? launch<true, false>(P, grid, status, st) : launch<false, false>(P, grid, status, st);
 }
@@ -777,7 +777,7 @@ cudaError_t proj3_fused(const Proj3Fused& a, bool split, unsigned* status, cudaS
   // Dc 16, D 4 (two a' tiles) 64 chains 14.3 / 14.3, 512 chains 32.0 / 33.2.
   // One tile of v leaves a stream idle, which costs where each chain would still have a CTA in the
   // one round of two per SM: cV 12, 192 chains 20.0 / 22.4; 152 chains 18.9 / 15.3, 580 chains 30.2 / 28.6.
-  if (P.n_at < 3 || (P.n_vt == 1 && a.batch > sms && a.batch <= 2 * sms)) return proj3_tiles(a, split, status, st);
+  if (P.n_at < 3 || (P.n_vt == 1 && a.batch > sms && a.batch <= 2 * sms)) return proj3_tiles(a, split, sms, status, st);
   if (all_full(P.op))
     return split ? launch_proj3<true, true>(P, grid, status, st) : launch_proj3<false, true>(P, grid, status, st);
   return split ? launch_proj3<true, false>(P, grid, status, st) : launch_proj3<false, false>(P, grid, status, st);

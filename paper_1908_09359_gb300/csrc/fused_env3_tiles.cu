@@ -415,15 +415,13 @@ __global__ void __launch_bounds__(kThreads, 2) env3_tile_kernel(const Env3Fused 
 }
 
 template <bool X3>
-cudaError_t launch(const Env3Fused& a, unsigned* status, cudaStream_t st) {
-  PV_CUDA(allow_smem(env3_tile_kernel<X3>, SMEM_BYTES, true));
-  int sms = 0;
-  PV_CUDA(sm_count(&sms));
+cudaError_t launch(const Env3Fused& a, int sms, unsigned* status, cudaStream_t st) {
+  static SmemLimit limit{SMEM_BYTES, true};
   const int ctas = 2 * sms;  // two resident CTAs per SM (104 KB shared memory, 128 registers x 256 threads each)
   const long long units = (long long)a.batch * ((a.cT2 + kAT - 1) / kAT);
   if (units > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = (int)(units < ctas ? units : ctas);
-  return launch_early(env3_tile_kernel<X3>, grid, kThreads, SMEM_BYTES, st, a, status);
+  return launch_large(limit, true, env3_tile_kernel<X3>, grid, kThreads, SMEM_BYTES, st, a, status);
 }
 
 // ------------------------------------------------------------ optimal site of the fit
@@ -699,25 +697,23 @@ __global__ void __launch_bounds__(kThreads, 2) proj3_tile_kernel(const Proj3Fuse
 }
 
 template <bool X3>
-cudaError_t launch_proj3(const Proj3Fused& a, unsigned* status, cudaStream_t st) {
-  PV_CUDA(allow_smem(proj3_tile_kernel<X3>, P_SMEM_BYTES, true));
-  int sms = 0;
-  PV_CUDA(sm_count(&sms));
+cudaError_t launch_proj3(const Proj3Fused& a, int sms, unsigned* status, cudaStream_t st) {
+  static SmemLimit limit{P_SMEM_BYTES, true};
   const int ctas = 2 * sms;
   const long long units = (long long)a.batch * ((a.cV + kPV - 1) / kPV);
   if (units > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = (int)(units < ctas ? units : ctas);
-  return launch_early(proj3_tile_kernel<X3>, grid, kThreads, P_SMEM_BYTES, st, a, status);
+  return launch_large(limit, true, proj3_tile_kernel<X3>, grid, kThreads, P_SMEM_BYTES, st, a, status);
 }
 
 }  // namespace
 
-cudaError_t env3_tiles(const Env3Fused& a, bool split, unsigned* status, cudaStream_t st) {
-  return split ? launch<true>(a, status, st) : launch<false>(a, status, st);
+cudaError_t env3_tiles(const Env3Fused& a, bool split, int sms, unsigned* status, cudaStream_t st) {
+  return split ? launch<true>(a, sms, status, st) : launch<false>(a, sms, status, st);
 }
 
-cudaError_t proj3_tiles(const Proj3Fused& a, bool split, unsigned* status, cudaStream_t st) {
-  return split ? launch_proj3<true>(a, status, st) : launch_proj3<false>(a, status, st);
+cudaError_t proj3_tiles(const Proj3Fused& a, bool split, int sms, unsigned* status, cudaStream_t st) {
+  return split ? launch_proj3<true>(a, sms, status, st) : launch_proj3<false>(a, sms, status, st);
 }
 
 }  // namespace pv

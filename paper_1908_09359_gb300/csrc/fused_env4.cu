@@ -338,10 +338,10 @@ __global__ void __launch_bounds__(kThreads, 2) env4_fused_kernel(const Env4Fused
 
 template <bool X3>
 cudaError_t launch(const Env4Fused& a, unsigned* status, cudaStream_t st) {
-  PV_CUDA(allow_smem(env4_fused_kernel<X3>, SMEM_BYTES, true));  // two CTAs per SM
+  static SmemLimit limit{SMEM_BYTES, true};  // two CTAs per SM
   const long long blocks = (long long)a.batch * ((a.cT2 + kAT - 1) / kAT);
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-  return launch_early(env4_fused_kernel<X3>, (unsigned)blocks, kThreads, SMEM_BYTES, st, a, status);
+  return launch_large(limit, true, env4_fused_kernel<X3>, (unsigned)blocks, kThreads, SMEM_BYTES, st, a, status);
 }
 
 }  // namespace

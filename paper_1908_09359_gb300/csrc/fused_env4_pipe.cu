@@ -459,8 +459,8 @@ void set_site(PipeOp& o, const float* base, long long slot, int nl, long long sl
 
 template <bool X3>
 cudaError_t launch(const Plan4& P, int grid, unsigned* status, cudaStream_t st) {
-  PV_CUDA(allow_smem(env4_pipe_kernel<X3>, SMEM_BYTES));
-  return launch_early(env4_pipe_kernel<X3>, grid, kThreads, SMEM_BYTES, st, P, status);
+  static SmemLimit limit{SMEM_BYTES, false};
+  return launch_large(limit, true, env4_pipe_kernel<X3>, grid, kThreads, SMEM_BYTES, st, P, status);
 }
 
 }  // namespace

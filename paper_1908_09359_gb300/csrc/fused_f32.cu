@@ -408,8 +408,10 @@ cudaError_t env3_f32(const Env3Fused& a, float* out1, bool rev2, bool rev3, cons
   int sms = 0;
   PV_CUDA(sm_count(&sms));
   auto* kernel = mid.p ? env3_f32_kernel<true> : env3_f32_kernel<false>;
-  if (smem > 48 * 1024) PV_CUDA(allow_smem(kernel, kMaxSmem));
-  return launch_early(kernel, (unsigned)blocks, threads_for(tasks > tasks2 ? tasks : tasks2, smem, blocks, sms), smem, st, a, out1, rev2, rev3, mid);
+  const int threads = threads_for(tasks > tasks2 ? tasks : tasks2, smem, blocks, sms);
+  if (smem <= 48 * 1024) return launch_early(kernel, (unsigned)blocks, threads, smem, st, a, out1, rev2, rev3, mid);
+  static SmemLimit limit[2] = {{kMaxSmem, false}, {kMaxSmem, false}};
+  return launch_large(limit[mid.p != nullptr], true, kernel, (unsigned)blocks, threads, smem, st, a, out1, rev2, rev3, mid);
 }
 
 static bool several(const Env4Outs& o) { return (o.p[0] != nullptr) + (o.p[1] != nullptr) + (o.p[2] != nullptr) + (o.p[3] != nullptr) > 1; }
@@ -451,13 +453,15 @@ cudaError_t env4_f32(const Env4Fused& a, const Env4Outs& outs, bool rev, cudaStr
   if (g_dry_run || a.batch <= 0) return cudaSuccess;
   int off[7];
   const int smem = layout4(a, several(outs), off) * 4;
-  if (smem > 48 * 1024) PV_CUDA(allow_smem(env4_f32_kernel, kMaxSmem));
   const long long blocks = (long long)a.batch * ((a.cT2 + kTA - 1) / kTA);
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int tasks = a.D2l * a.cB * ((a.D1r * a.Dd1 + 3) / 4);
   int sms = 0;
   PV_CUDA(sm_count(&sms));
-  return launch_early(env4_f32_kernel, (unsigned)blocks, threads_for(tasks, smem, blocks, sms), smem, st, a, outs, several(outs), rev);
+  const int threads = threads_for(tasks, smem, blocks, sms);
+  if (smem <= 48 * 1024) return launch_early(env4_f32_kernel, (unsigned)blocks, threads, smem, st, a, outs, several(outs), rev);
+  static SmemLimit limit{kMaxSmem, false};
+  return launch_large(limit, true, env4_f32_kernel, (unsigned)blocks, threads, smem, st, a, outs, several(outs), rev);
 }
 
 }  // namespace pv

@@ -439,9 +439,8 @@ cudaError_t qr_pos_batched(const float* Y, long long bsY, long long yrs, long lo
   const size_t smem = (size_t)2 * rows * cols * sizeof(float);
   constexpr size_t kMost = kCtaSmem - kQrMaxCols * (sizeof(float) + sizeof(int)) - kQrThreads / 32 * sizeof(float);
   if (smem > kMost) return cudaErrorInvalidValue;
-  PV_CUDA(allow_smem(qr_pos_kernel, kMost));
-  qr_pos_kernel<<<batch, kQrThreads, smem, st>>>(Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols);
-  return cudaGetLastError();
+  static SmemLimit limit{kMost, false};
+  return launch_large(limit, false, qr_pos_kernel, batch, kQrThreads, smem, st, Y, bsY, yrs, ycs, Q, bsQ, qrs, qcs, rows, cols);
 }
 
 }  // namespace pv

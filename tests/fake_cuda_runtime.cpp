@@ -29,7 +29,7 @@ std::map<const void*, std::string> names;
 std::map<std::pair<int, const void*>, size_t> limits;  // dynamic shared memory, by device and kernel
 std::vector<Launch> launches;
 cudaError_t pending = cudaSuccess;
-int device = 0, refuse_limits = 0;
+int device = 0, refuse_limits = 0, limits_set = 0;
 bool capture_elsewhere = false;
 
 cudaError_t set(cudaError_t e) {
@@ -92,6 +92,7 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
   return launch(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, early);
 }
 cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
+  ++limits_set;
   if (refuse_limits > 0) {
     --refuse_limits;
     return set(cudaErrorNotReady);
@@ -160,6 +161,7 @@ void fake_reset_device() {
 void fake_refuse_limits(int n) { refuse_limits = n; }
 void fake_capture_elsewhere(int on) { capture_elsewhere = on; }
 void fake_pending(int e) { pending = (cudaError_t)e; }
+int fake_limits_set() { return limits_set; }
 int fake_launches() { return (int)launches.size(); }
 void fake_clear() { launches.clear(); }
 const char* fake_name(int i) { return launches[i].name.c_str(); }

@@ -134,6 +134,10 @@ def test_shared_memory_is_granted_on_whatever_device_is_current(fake, what):
         fake.fake_clear()
 
     runs()
+    before = fake.fake_limits_set()
+    runs()                      # host time: asked for once, not at every launch
+    assert fake.fake_limits_set() == before
+    grids.pop()
     fake.fake_device(1)         # another device, with half the SMs
     runs()
     assert grids[1] <= grids[0]
@@ -174,8 +178,10 @@ def test_a_refused_launch_is_reported_once(fake, launch):
 
 def test_an_error_of_the_callers_stays_the_callers(fake):
     """Pending from before the call: neither reported as the launch's nor dropped."""
+    large = (24, 24, 24, 24, 6, 6, 6, 6)
+    assert noalloc(fake, 8, large) == OK  # (a launch refused after a device reset would take its place)
     fake.fake_pending(999)
-    assert fake.host_dot(100, 4) == OK and noalloc(fake, 8, (24, 24, 24, 24, 6, 6, 6, 6)) == OK
+    assert fake.host_dot(100, 4) == OK and noalloc(fake, 8, large) == OK
     assert fake.cudaPeekAtLastError() == 999
 
 
