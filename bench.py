@@ -49,11 +49,11 @@ FP32_ALU_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 # includes) hashed to `source_sha`, per chain of that capture; the bench reports it only while
 # the source is unchanged.
 NCU_TRAFFIC = {
-    "fused4": {"bytes_per_chain": (206.821120e6 + 98.171392e6) / 512,
-               "source": "paper_1908_09359_gb300/csrc/fused_env4_pipe.cu", "source_sha": "1838eb19c1f657e2",
+    "fused4": {"bytes_per_chain": (205.779712e6 + 98.166272e6) / 512,
+               "source": "paper_1908_09359_gb300/csrc/fused_env4_pipe.cu", "source_sha": "52f565b0e02449f0",
                "summary": "profiles/fused4_env4_bulk_peps24x24.md"},
-    "fused3": {"bytes_per_chain": (210.121216e6 + 44.955136e6) / 2048,
-               "source": "paper_1908_09359_gb300/csrc/fused_env3.cu", "source_sha": "49eca88d80eb98a0",
+    "fused3": {"bytes_per_chain": (210.055680e6 + 44.630016e6) / 2048,
+               "source": "paper_1908_09359_gb300/csrc/fused_env3.cu", "source_sha": "65103bb92e1ed7f9",
                "summary": "profiles/fused3_env3_bulk_peps24x24.md"},
 }
 
