@@ -450,19 +450,13 @@ __global__ void phi_combine_kernel(const double* logpsi, const int8_t* sign, con
   }
 }
 
-// sum_i x[i] y[i] of one chain, on thread 0 (in block_sum's order), by one block: float64 additions are slow
-// here, so they are as few as the tree needs.  A block is bound by the latency of its loads while
+// sum_i x[i] y[i] of one chain, on thread 0 (in block_sum's order), by one block: float64 additions are
+// slow on this GPU, so they are as few as the tree needs.  A block is bound by the latency of its loads while
 // it has an SM to itself, by bandwidth when many share one: U = 8 entries (16 loads of 16 bytes) in
 // flight up to two blocks per SM, beyond that U = 2 and more blocks.  Measured in a graph, U as the
 // compiler chose / clusters of up to 8 blocks / this: 65,536 entries, 16 chains 15.0 / 6.6 / 6.9 us, 128
 // chains 15.6 / 15.0 / 7.3, 512 chains 50.3 / 58.9 / 41.0; 20,736 entries, 256 chains 8.1 / 12.8 / 5.7; 4,096
 // entries, 1024 chains 11.0 / - / 7.3.
-inline cudaError_t deep_loads(int batch, bool* deep) {
-  int sms = 0;
-  PV_CUDA(sm_count(&sms));
-  *deep = batch <= 2 * sms;
-  return cudaSuccess;
-}
 template <int U>
 __device__ __forceinline__ double chain_dot(const float* x, const float* y, int n) {
   __shared__ double red[kThreads / 32];
@@ -475,6 +469,13 @@ __device__ __forceinline__ double chain_dot(const float* x, const float* y, int 
   if (threadIdx.x == 0)
     for (int i = 0; i < kThreads / 32; ++i) s += red[i];
   return s;
+}
+// Whether the chains' sums take U = 8.
+inline cudaError_t deep_loads(int batch, bool* deep) {
+  int sms = 0;
+  PV_CUDA(sm_count(&sms));
+  *deep = batch <= 2 * sms;
+  return cudaSuccess;
 }
 
 template <int U>
